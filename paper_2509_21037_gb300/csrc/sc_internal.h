@@ -176,6 +176,7 @@ struct sc_ctx {
   // per wave, launch groups by variant (index 0 = FP64, 3..7 = digits): first item, count
   struct WaveGroups {
     int64_t trsm[sc::kNumVariants][2] = {}, syrk[sc::kNumVariants][2] = {}, sblk[sc::kNumVariants][2] = {};
+    int syrk_ctas = 1;   // FP64 group: CTAs per SYRK task (sc_plan.cpp)
   };
   std::vector<WaveGroups> waves;
   std::vector<int32_t> sub_wave;     // wave of every subdomain

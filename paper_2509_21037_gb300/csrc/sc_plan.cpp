@@ -541,6 +541,18 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       g[1]++;
     }
   };
+  // total and longest cost of every wave's FP64 group
+  auto each_group = [&](const std::vector<double> &cost, const std::vector<int8_t> &var,
+                        const std::vector<int32_t> &wave, const std::vector<int32_t> &o, auto set) {
+    std::vector<double> total(ctx->waves.size(), 0.0), longest(ctx->waves.size(), 0.0);
+    for (int32_t k : o) {
+      if (var[k] != 0) continue;
+      total[wave[k]] += cost[k];
+      longest[wave[k]] = std::max(longest[wave[k]], cost[k]);
+    }
+    for (size_t w = 0; w < total.size(); ++w)
+      if (total[w] > 0.0) set(ctx->waves[w], total[w], longest[w]);
+  };
   {
     auto o = order_by(trsm_cost, trsm_var, trsm_wave);
     // The TRSM of a batch is about one wave of resident CTAs, so what the launch
@@ -563,6 +575,14 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
   {
     auto o = order_by(syrk_cost, syrk_var, syrk_wave);
     groups(syrk_var, syrk_wave, o, 1);
+    // CTAs per SYRK task: one as long as the longest task (a CTA's warps share it evenly) takes at
+    // most a quarter of an SM's share of the whole, else 4 or 8.  GB300, ms at 1 / 4 / 8: 64 heat cubes
+    // 30.3 / 30.7 / 31.3 (rule: 1), 8 elasticity cubes 6.46 / 6.49 / 6.57 (1), 36 plane squares
+    // 0.196 / 0.153 / 0.155 (4), one square 0.031 / 0.018 / 0.014 (8).
+    each_group(syrk_cost, syrk_var, syrk_wave, o, [&](sc_ctx::WaveGroups &g, double total, double longest) {
+      const double r = longest * kGridSMs / total;
+      g.syrk_ctas = r <= 0.25 ? 1 : r <= 1.0 ? 4 : 8;
+    });
     std::vector<SyrkTask> t2(syrk.size());
     for (size_t k = 0; k < o.size(); ++k) t2[k] = syrk[o[k]];
     syrk.swap(t2);
