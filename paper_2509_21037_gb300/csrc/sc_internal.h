@@ -122,6 +122,7 @@ struct PlanPtrs {
   const ApplyTask *apply_tasks;
   const int32_t *active_cols; // global column indices whose reciprocal diagonal is needed
   const int32_t *cuts;       // per supernode and 32-row block: sorted columns >= cut are zero there
+  const int32_t *seed_ptr;   // first seed of every sorted column of the batch, and the end
   const int32_t *sblk;       // (active supernode, 32-row block) pairs, for the split-precision packing
 };
 
@@ -147,6 +148,7 @@ struct PlanHeader {
   int64_t n_sns, n_trsm, n_syrk, n_apply, n_cols, n_active_cols;
   uint64_t sec_off[kNumSections];   // subs sns lcp rmap trsm trsm_list syrk syrk_list seeds perm lambda apply active cuts sblk
   uint64_t sec_bytes[kNumSections];
+  uint64_t seed_ptr_off, seed_ptr_bytes;   // one section more, after the numbered ones
 };
 constexpr size_t kHeaderBytes = 512;
 static_assert(sizeof(PlanHeader) <= kHeaderBytes, "plan header must fit its reserved bytes");
@@ -176,7 +178,7 @@ struct sc_ctx {
   // per wave, launch groups by variant (index 0 = FP64, 3..7 = digits): first item, count
   struct WaveGroups {
     int64_t trsm[sc::kNumVariants][2] = {}, syrk[sc::kNumVariants][2] = {}, sblk[sc::kNumVariants][2] = {};
-    int syrk_ctas = 1;   // FP64 group: CTAs per SYRK task (sc_plan.cpp)
+    int trsm_cols = 16, syrk_ctas = 1;   // FP64 group: columns per TRSM warp, CTAs per SYRK task (sc_plan.cpp)
   };
   std::vector<WaveGroups> waves;
   std::vector<int32_t> sub_wave;     // wave of every subdomain
@@ -184,7 +186,7 @@ struct sc_ctx {
   int64_t n_dual = 0;
   std::vector<uint8_t> blob;     // plan tables, 256-byte aligned sections
   sc::Section s_subs, s_sns, s_lcp, s_rmap, s_trsm, s_trsm_list, s_syrk, s_syrk_list, s_seeds,
-      s_perm, s_lambda, s_apply, s_active, s_cuts, s_sblk;
+      s_perm, s_lambda, s_apply, s_active, s_cuts, s_sblk, s_seed_ptr;
   int64_t n_sns = 0, n_trsm = 0, n_syrk = 0, n_apply = 0, n_cols = 0, n_active_cols = 0, n_sblk = 0;
   std::vector<int64_t> F_offsets, L_offsets;
   std::vector<sc::SubFeat> sub_feat;    // per subdomain, in batch order

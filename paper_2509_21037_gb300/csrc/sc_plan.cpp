@@ -242,7 +242,7 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
   std::vector<SyrkTask> syrk;
   std::vector<int32_t> syrk_list;
   std::vector<Seed> seeds;
-  std::vector<int32_t> perm, lam;
+  std::vector<int32_t> perm, lam, seed_ptr;
   std::vector<ApplyTask> apply;
   std::vector<int32_t> active_cols;
   std::vector<int32_t> cuts;
@@ -374,11 +374,9 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       }
     }
     // seeds, by sorted column
-    std::vector<int32_t> seed_ptr(m + 1, 0);
-    int32_t seed_base = (int32_t)seeds.size();
     for (int32_t q = 0; q < m; ++q) {
       int32_t j = S.perm_cols[q];
-      seed_ptr[q] = (int32_t)seeds.size();
+      seed_ptr.push_back((int32_t)seeds.size());
       for (int32_t e = D.Bt_colptr[j]; e < D.Bt_colptr[j + 1]; ++e) {
         int32_t r = D.Bt_rowind[e];
         int32_t s = S.snode_of[r];
@@ -389,8 +387,8 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
         seeds.push_back(sdd);
       }
     }
-    seed_ptr[m] = (int32_t)seeds.size();
-    (void)seed_base;
+    seed_ptr.push_back((int32_t)seeds.size());
+    const int32_t *sub_seed_ptr = seed_ptr.data() + col_total;
     // chunk lists
     const int32_t nchunk = nt;
     std::vector<std::vector<int32_t>> clist(nchunk);
@@ -405,8 +403,8 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       t.w = std::min(kChunk, m - t.c_lo);
       t.list_off = (int32_t)trsm_list.size();
       t.list_len = (int32_t)clist[q].size();
-      t.seed_lo = seed_ptr[t.c_lo];
-      t.seed_hi = seed_ptr[t.c_lo + t.w];
+      t.seed_lo = sub_seed_ptr[t.c_lo];
+      t.seed_hi = sub_seed_ptr[t.c_lo + t.w];
       double cost = 0, exec = 0;
       for (int32_t s : clist[q]) {
         trsm_list.push_back(gidx[s]);
@@ -517,9 +515,11 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       f.y_doubles = (double)(y_all + y_total - y0);
       ctx->sub_feat.push_back(f);
     }
+    seed_ptr.pop_back();         // the next subdomain's first column continues there
     col_total += m;
     lcp_total += n;
   }
+  seed_ptr.push_back((int32_t)seeds.size());
   // grouped by wave and variant (one launch per group), largest tasks first
   // inside a group: the block scheduler hands out CTAs roughly in index order
   auto order_by = [](const std::vector<double> &cost, const std::vector<int8_t> &var,
@@ -568,6 +568,17 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       g0 = g1;
     }
     groups(trsm_var, trsm_wave, o, 0);
+    // Columns per warp of the FP64 TRSM.  Wide parts waste the fewest lanes in the
+    // triangles, narrow ones shorten the longest part, which one warp works through alone
+    // on a sub-partition's FP64 unit.  The widest whose longest part is at most half of a
+    // sub-partition's share of the whole (4 per SM) is taken.  GB300, ms at 1 / 2 / 4 / 8 / 16
+    // columns: 64 heat cubes 22.9 / 19.8 / 18.4 / 17.9 / 17.4 (rule: 16), 8 elasticity cubes
+    // 7.80 / 7.78 / 10.7 / 15.3 / 33.7 (2), 36 plane squares 0.355 / 0.280 / 0.299 / 0.425 / 0.82 (2),
+    // one square 0.031 / 0.035 / 0.050 / 0.065 / 0.10 (1).
+    each_group(trsm_cost, trsm_var, trsm_wave, o, [&](sc_ctx::WaveGroups &g, double total, double longest) {
+      g.trsm_cols = 16;
+      while (g.trsm_cols > 1 && longest * g.trsm_cols / kChunk > 0.5 * total / (4 * kGridSMs)) g.trsm_cols /= 2;
+    });
     std::vector<TrsmTask> t2(trsm.size());
     for (size_t k = 0; k < o.size(); ++k) t2[k] = trsm[o[k]];
     trsm.swap(t2);
@@ -617,6 +628,7 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
   add_section(ctx->blob, ctx->s_active, active_cols);
   add_section(ctx->blob, ctx->s_cuts, cuts);
   add_section(ctx->blob, ctx->s_sblk, sblk);
+  add_section(ctx->blob, ctx->s_seed_ptr, seed_ptr);
   ctx->blob.resize((ctx->blob.size() + 255) & ~size_t(255));
   ctx->n_sns = (int64_t)sns.size();
   ctx->n_trsm = (int64_t)trsm.size();
@@ -638,6 +650,8 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
                                          &ctx->s_perm, &ctx->s_lambda, &ctx->s_apply, &ctx->s_active,
                                          &ctx->s_cuts, &ctx->s_sblk};
     for (int k = 0; k < kNumSections; ++k) { h.sec_off[k] = secs[k]->off; h.sec_bytes[k] = secs[k]->bytes; }
+    h.seed_ptr_off = ctx->s_seed_ptr.off;
+    h.seed_ptr_bytes = ctx->s_seed_ptr.bytes;
     std::memcpy(ctx->blob.data(), &h, sizeof(h));
   }
 
@@ -691,6 +705,7 @@ sc::PlanPtrs sc_ctx::ptrs() const {
   p.apply_tasks = reinterpret_cast<const ApplyTask *>(b + s_apply.off);
   p.active_cols = reinterpret_cast<const int32_t *>(b + s_active.off);
   p.cuts = reinterpret_cast<const int32_t *>(b + s_cuts.off);
+  p.seed_ptr = reinterpret_cast<const int32_t *>(b + s_seed_ptr.off);
   p.sblk = reinterpret_cast<const int32_t *>(b + s_sblk.off);
   return p;
 }
