@@ -17,8 +17,8 @@
  * Work: only the supernodes of L on the elimination-tree paths from B_i^T's
  * rows to the root are visited (the forward solve's right-hand side is zero
  * elsewhere, and the backward solve is read only at B_i^T's rows, which depend
- * on their ancestors alone).  A subdomain is solved by one CTA or, when large,
- * by a cluster of 8 CTAs; the supernodes of one etree level are solved
+ * on their ancestors alone).  A piece of a subdomain's tree is solved by one
+ * CTA (sci_options); the supernodes of one etree level are solved
  * concurrently by the group's warps, 32-column blocks at a time (warp-level
  * diagonal-block solve, coalesced panel updates), and the few large
  * separators at the top of the tree by the whole group.
@@ -67,22 +67,22 @@ typedef struct {
   int64_t n_cluster_subdomains; /* subdomains solved by a whole 8-CTA cluster */
 } sci_sizes;
 
-/* cluster_min_work: subdomains with at least this many visited entries of L
- * are solved by a thread-block cluster of 8 CTAs (8 SMs' FP64 pipes; cluster
+/* By default (a NULL options pointer, or cluster_min_work = -1 and pairs not 1)
+ * every subdomain's visited tree is cut into up to four tiers of subtrees, one
+ * CTA to a piece, one launch per tier and direction, so that a batch of
+ * fewer subdomains than SMs still fills the GPU.
+ * cluster_min_work >= 0: subdomains with at least this many visited entries of
+ * L are solved by a thread-block cluster of 8 CTAs (8 SMs' FP64 pipes; cluster
  * barriers between levels, distributed shared memory for the reductions),
- * the others by one CTA each (packed 8 to a cluster).  -1 (or a NULL options
- * pointer) selects more than 2 x (visited entries of the batch) /
- * min(304, nsub): twice an even share of the CTAs the batch can occupy (a
- * GB300 keeps 304 resident).  Clusters shorten a heavy tail of a few large
- * subdomains; on a batch of similar subdomains they cost more (cluster
- * barriers, L1-bypassing reads of x) than they give.  0 puts every subdomain
- * on a cluster. */
+ * the others by one CTA each (packed 8 to a cluster).  0 puts every subdomain
+ * on a cluster.  -1 with pairs = 1: more than 2 x (visited entries of the batch) /
+ * min(152, nsub) entries. */
 /* pairs: 1 solves each subdomain below cluster_min_work whose visited etree
  * splits on a pair of CTAs: the subtrees below the first node with two or
  * more substantial visited subtrees are dealt to the two CTAs (about half the
  * work each), which solve them at the same time; the chain above runs on the
- * first CTA; three cluster barriers per call.  0 (automatic) and -1: one CTA
- * per subdomain (on GB300 the pair form measured slower on the 64-subdomain
+ * first CTA; three cluster barriers per call.  0 (automatic) and -1: no pairs
+ * (on GB300 the pair form measured slower on the 64-subdomain
  * heat batch: the per-level chains, not the subtrees, bound the solve).
  * reserved: 0. */
 typedef struct {

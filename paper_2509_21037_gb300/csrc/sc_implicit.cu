@@ -8,8 +8,10 @@
 // parent is at least one level above each child), B^T grouped by row for the
 // gather and by entry for the scatter.
 //
-// Device side: one CTA per subdomain (largest first).  Forward solve level by
-// level upwards, backward solve level by level downwards, the warps sharing
+// Device side: a tiered schedule by default (see "the tiered schedule" below:
+// 64 heat cubes 1.45 -> 0.75 ms); clusters or CTA pairs where the options ask
+// for them, then one launch with one CTA per subdomain otherwise.
+// Forward solve level by level upwards, backward solve level by level downwards, the warps sharing
 // the supernodes of a level; a barrier between levels.  A warp solves its
 // supernode in 32-column blocks:
 //   forward   the block's triangle with lane = row (32 shuffle steps, the
@@ -33,6 +35,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <limits>
 #include <new>
 
 #include <algorithm>
@@ -99,6 +102,13 @@ struct IItem {
 };
 static_assert(sizeof(IItem) == 40, "IItem layout");
 
+// A piece of a subdomain's visited tree for the tiered schedule: a set of whole subtrees of what its
+// tier is left with, solved by one CTA (levels and scatter entries as in ISub).
+struct IPiece {
+  int32_t sub, lev_lo, n_lev, s_lo, s_hi, pad;
+};
+
+constexpr int kTiers = 4;
 constexpr int kSections = 8;
 struct IHeader {
   uint32_t magic;     // 'SCIP'
@@ -106,6 +116,8 @@ struct IHeader {
   int32_t nsub, pad;
   int64_t n_sn, n_levptr, n_rows, n_grow, n_gent, n_sent, n_items;
   uint64_t sec_off[kSections];   // subs sns levptr rows grow gent sent items
+  uint64_t piece_off;            // one section more: the pieces, tier by tier, largest first
+  int64_t n_pieces;
 };
 constexpr size_t kIHeaderBytes = 256;
 static_assert(sizeof(IHeader) <= kIHeaderBytes, "implicit plan header");
@@ -119,6 +131,7 @@ struct IPtrs {
   const IEnt *gent;
   const ISEnt *sent;
   const IItem *items;
+  const IPiece *pieces;
   int64_t rd_off;      // doubles from a subdomain's x to its reciprocal diagonals (workspace)
 };
 
@@ -151,9 +164,13 @@ __device__ __forceinline__ double forward_triangle(const double *__restrict__ L,
     o += nr - (kb + k) - 1;
   }
   double xi = lane < w ? ldx<CL>(xs + kb + lane) : 0.0;
+  // eight columns at a time with a branch in between: a step that is only predicated off would
+  // take its place in the chain and on the FP64 pipe (columns past w: lv = inv = 0, x stays)
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    if (k < w) {   // uniform
+  for (int k0 = 0; k0 < 32; k0 += 8) {
+    if (k0 >= w) break;   // uniform
+#pragma unroll
+    for (int k = k0; k < k0 + 8; ++k) {
       const double yk = __shfl_sync(kFull, xi, k) * __shfl_sync(kFull, inv, k);
       xi = lane == k ? yk : fma(-lv[k], yk, xi);
     }
@@ -173,7 +190,6 @@ __device__ __forceinline__ void forward_panel_chunk(const double *__restrict__ L
   const int t = t0 + lane;
   const bool ok = t < nr;
   double lv[32];
-#pragma unroll
   // entry (t, c) of the panel at col_off(c) + t - c, and col_off(c + 1) = col_off(c) + nr - c
   int o = col_off(kb, nr) + (t - kb);
 #pragma unroll
@@ -181,10 +197,17 @@ __device__ __forceinline__ void forward_panel_chunk(const double *__restrict__ L
     lv[k] = (k < w && ok) ? L[o] : 0.0;
     o += nr - (kb + k) - 1;
   }
-  double acc = 0.0;
+  double acc = 0.0, acc1 = 0.0;
 #pragma unroll
-  for (int k = 0; k < 32; ++k)
-    if (k < w) acc = fma(lv[k], ys[k], acc);
+  for (int k0 = 0; k0 < 32; k0 += 8) {
+    if (k0 >= w) break;   // uniform; lv = 0 past w
+#pragma unroll
+    for (int k = k0; k < k0 + 8; k += 2) {
+      acc = fma(lv[k], ys[k], acc);
+      acc1 = fma(lv[k + 1], ys[k + 1], acc1);
+    }
+  }
+  acc += acc1;
   if (!ok) return;
   if (t < ns) xs[t] = ldx<CL>(xs + t) - acc;
   else atomicAdd(x + R[t - ns], -acc);
@@ -200,9 +223,16 @@ __device__ __forceinline__ void backward_panel_chunk(const double *__restrict__ 
   const double zt = ok ? (t < ns ? ldx<CL>(xs + t) : ldx<CL>(x + R[t - ns])) : 0.0;
   int o = col_off(kb, nr) + (t - kb);
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    if (k < w && ok) acc[k] = fma(L[o], zt, acc[k]);
-    o += nr - (kb + k) - 1;
+  for (int k0 = 0; k0 < 32; k0 += 8) {
+    if (k0 >= w) break;   // uniform
+    double l[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      l[k] = (k0 + k < w && ok) ? L[o] : 0.0;
+      o += nr - (kb + k0 + k) - 1;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k0 + k] = fma(l[k], zt, acc[k0 + k]);
   }
 }
 
@@ -222,27 +252,35 @@ __device__ __forceinline__ double transpose_reduce(double (&acc)[32], int lane) 
   return acc[0];
 }
 
+// The same over kLanes lanes for the first P columns: a transpose-reduce over groups of P lanes, then a
+// butterfly across the groups.
+template <int P, int kLanes, int N>
+__device__ __forceinline__ double transpose_reduce_p(double (&acc)[N], int lane) {
+#pragma unroll
+  for (int h = P / 2; h >= 1; h >>= 1) {
+    const bool up = (lane & h) != 0;
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const double send = up ? acc[j] : acc[j + h];
+      const double keep = up ? acc[j + h] : acc[j];
+      acc[j] = keep + __shfl_xor_sync(kFull, send, h);
+    }
+  }
+  double v = acc[0];
+#pragma unroll
+  for (int m = P; m < kLanes; m <<= 1) v += __shfl_xor_sync(kFull, v, m);
+  return v;
+}
+
 // The same for the first w < 32 columns (acc[k] = 0 for k >= w): a
 // transpose-reduce over groups of P lanes (P the power of two >= w), then a
 // butterfly across the 32 / P groups: P - 1 + 5 - log2 P additions instead of 31.
 __device__ __forceinline__ double transpose_reduce_w(double (&acc)[32], int lane, int w) {
   if (w > 16) return transpose_reduce(acc, lane);
-  const int P = w <= 1 ? 1 : w <= 2 ? 2 : w <= 4 ? 4 : w <= 8 ? 8 : 16;
-#pragma unroll
-  for (int h = 8; h >= 1; h >>= 1) {
-    if (h < P) {   // uniform
-      const bool up = (lane & h) != 0;
-#pragma unroll
-      for (int j = 0; j < h; ++j) {
-        const double send = up ? acc[j] : acc[j + h];
-        const double keep = up ? acc[j + h] : acc[j];
-        acc[j] = keep + __shfl_xor_sync(kFull, send, h);
-      }
-    }
-  }
-  double v = acc[0];
-  for (int m = P; m < 32; m <<= 1) v += __shfl_xor_sync(kFull, v, m);
-  return v;
+  if (w > 8) return transpose_reduce_p<16, 32>(acc, lane);
+  if (w > 4) return transpose_reduce_p<8, 32>(acc, lane);
+  if (w > 2) return transpose_reduce_p<4, 32>(acc, lane);
+  return transpose_reduce_p<2, 32>(acc, lane);
 }
 
 // Backward triangle of one block (one warp, lane = column): z = L_bb^{-T} rhs, written to x.
@@ -256,11 +294,12 @@ __device__ __forceinline__ void backward_triangle(const double *__restrict__ L, 
 #pragma unroll
   for (int i = 0; i < 32; ++i) lc[i] = (i > lane && i < w) ? pc[i] : 0.0;
 #pragma unroll
-  for (int i = 31; i >= 0; --i) {
-    if (i < w) {   // uniform
-      if (lane == i) rhs *= inv;
-      const double zi = __shfl_sync(kFull, rhs, i);
-      rhs = fma(-lc[i], zi, rhs);
+  for (int i0 = 24; i0 >= 0; i0 -= 8) {
+    if (i0 >= w) continue;   // uniform
+#pragma unroll
+    for (int i = i0 + 7; i >= i0; --i) {      // columns past w: rhs = inv = lc = 0
+      const double zi = __shfl_sync(kFull, rhs * inv, i);
+      rhs = lane == i ? zi : fma(-lc[i], zi, rhs);
     }
   }
   if (lane < w) xs[kb + lane] = rhs;
@@ -347,113 +386,130 @@ __device__ void backward_warp(const ISn &sn, const double *__restrict__ Lv, cons
 // zero, so they add nothing.  valid = false: the half has no supernode.  A
 // supernode of at most 16 columns is one block, and every row below it is a
 // pruned row (an ancestor's).
-template <bool CL>
-__device__ void forward_half(const ISn &sn, bool valid, const double *__restrict__ Lv,
-                             const int32_t *__restrict__ rows, double *x, double *ys, int64_t rd_off, int lane) {
-  const int hl = lane & 15, h = lane >> 4;
-  const int ns = valid ? sn.ns : 0, nr = valid ? sn.ns + sn.rs : 0;
-  const double *L = Lv + (valid ? sn.lval : 0);
-  const int32_t *R = rows + (valid ? sn.rows_off : 0);
-  double *xs = x + (valid ? sn.c0 : 0);
-  const int wmax = max(ns, __shfl_xor_sync(kFull, ns, 16));
+// WM: the columns of the wider of the two, rounded up to a power of two -- a constant, so that no step of the
+// chain and no multiply-add is there only to be predicated off (most supernodes have one to four columns;
+// with every loop run to 16 a level of them took 4 us instead of 2).
+template <bool CL, int WM>
+__device__ __forceinline__ void forward_half_w(int ns, int nr, const double *__restrict__ L,
+                                               const int32_t *__restrict__ R, double *xs, double *x,
+                                               int64_t rd_off, int lane) {
+  const int hl = lane & 15;
   const int nch = (nr - ns + 15) >> 4, chmax = max(nch, __shfl_xor_sync(kFull, nch, 16));
+  int t = ns + hl;
+  int r = t < nr ? R[t - ns] : 0;                  // the first rows' indices and L entries, before the triangle
+  double lb[WM];
+  {
+    int o = t;
+#pragma unroll
+    for (int k = 0; k < WM; ++k) {
+      lb[k] = (k < ns && t < nr) ? L[o] : 0.0;
+      o += nr - k - 1;
+    }
+  }
   const double inv = hl < ns ? ldx<CL>(xs + rd_off + hl) : 0.0;
   // lane i: L(i, k) for k < i, entry (i - k) of column k (offsets stepped column to column)
-  double lv[16];
+  double lv[WM];
   int o = hl;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
+  for (int k = 0; k < WM; ++k) {
     lv[k] = (k < ns && k < hl && hl < ns) ? L[o] : 0.0;
     o += nr - k - 1;
   }
   double xi = hl < ns ? ldx<CL>(xs + hl) : 0.0;
+  double y[WM];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    if (k < wmax) {   // uniform
-      const double yk = __shfl_sync(kFull, xi, k, 16) * __shfl_sync(kFull, inv, k, 16);
-      xi = hl == k ? yk : fma(-lv[k], yk, xi);
-    }
+  for (int k = 0; k < WM; ++k) {
+    y[k] = __shfl_sync(kFull, xi, k, 16) * __shfl_sync(kFull, inv, k, 16);
+    xi = hl == k ? y[k] : k + 1 < WM ? fma(-lv[k], y[k], xi) : xi;
   }
   if (hl < ns) xs[hl] = xi;
-  ys[16 * h + hl] = hl < ns ? xi : 0.0;
-  __syncwarp();
   for (int ch = 0; ch < chmax; ++ch) {
-    const int t = ns + 16 * ch + hl;
-    const bool ok = t < nr;
-    int oo = t;
     double acc = 0.0;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      if (k < wmax) {   // uniform
-        const double l = (k < ns && ok) ? L[oo] : 0.0;
-        acc = fma(l, ys[16 * h + k], acc);
+    for (int k = 0; k < WM; ++k) acc = fma(lb[k], y[k], acc);
+    if (t < nr) atomicAdd(x + r, -acc);
+    t += 16;
+    if (ch + 1 < chmax) {
+      r = t < nr ? R[t - ns] : 0;
+      int oo = t;
+#pragma unroll
+      for (int k = 0; k < WM; ++k) {
+        lb[k] = (k < ns && t < nr) ? L[oo] : 0.0;
+        oo += nr - k - 1;
       }
-      oo += nr - k - 1;
     }
-    if (ok) atomicAdd(x + R[t - ns], -acc);
   }
   __syncwarp();
 }
 
 template <bool CL>
-__device__ void backward_half(const ISn &sn, bool valid, const double *__restrict__ Lv,
-                              const int32_t *__restrict__ rows, double *x, int64_t rd_off, int lane) {
-  const int hl = lane & 15;
+__device__ void forward_half(const ISn &sn, bool valid, const double *__restrict__ Lv,
+                             const int32_t *__restrict__ rows, double *x, int64_t rd_off, int lane) {
   const int ns = valid ? sn.ns : 0, nr = valid ? sn.ns + sn.rs : 0;
   const double *L = Lv + (valid ? sn.lval : 0);
   const int32_t *R = rows + (valid ? sn.rows_off : 0);
   double *xs = x + (valid ? sn.c0 : 0);
   const int wmax = max(ns, __shfl_xor_sync(kFull, ns, 16));
+  if (wmax <= 1) forward_half_w<CL, 1>(ns, nr, L, R, xs, x, rd_off, lane);
+  else if (wmax <= 2) forward_half_w<CL, 2>(ns, nr, L, R, xs, x, rd_off, lane);
+  else if (wmax <= 4) forward_half_w<CL, 4>(ns, nr, L, R, xs, x, rd_off, lane);
+  else if (wmax <= 8) forward_half_w<CL, 8>(ns, nr, L, R, xs, x, rd_off, lane);
+  else forward_half_w<CL, 16>(ns, nr, L, R, xs, x, rd_off, lane);
+}
+
+template <bool CL, int WM>
+__device__ __forceinline__ void backward_half_w(int ns, int nr, const double *__restrict__ L,
+                                                const int32_t *__restrict__ R, double *xs, const double *x,
+                                                int64_t rd_off, int lane) {
+  const int hl = lane & 15;
   const int nch = (nr - ns + 15) >> 4, chmax = max(nch, __shfl_xor_sync(kFull, nch, 16));
-  double acc[16];
+  const double inv = hl < ns ? ldx<CL>(xs + rd_off + hl) : 0.0;
+  const double xo = hl < ns ? ldx<CL>(xs + hl) : 0.0;
+  // lane k: L(i, k) for i > k, entry (i - k) of its own column
+  const double *pc = L + (hl < ns ? col_off(hl, nr) - hl : 0);
+  double lc[WM];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) acc[k] = 0.0;
+  for (int i = 0; i < WM; ++i) lc[i] = (i > hl && i < ns) ? pc[i] : 0.0;
+  double acc[WM];
+#pragma unroll
+  for (int k = 0; k < WM; ++k) acc[k] = 0.0;
   for (int ch = 0; ch < chmax; ++ch) {
     const int t = ns + 16 * ch + hl;
     const bool ok = t < nr;
     const double zt = ok ? ldx<CL>(x + R[t - ns]) : 0.0;
     int oo = t;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      if (k < wmax && k < ns && ok) acc[k] = fma(L[oo], zt, acc[k]);
+    for (int k = 0; k < WM; ++k) {
+      const double l = (k < ns && ok) ? L[oo] : 0.0;
+      acc[k] = fma(l, zt, acc[k]);
       oo += nr - k - 1;
     }
   }
-  // sum of acc[k] over the half's lanes, lane k of the half ending with column k: a
-  // transpose-reduce over groups of P lanes (P the power of two >= wmax), then a butterfly
-  // across the half's 16 / P groups (xor distances below 16 stay inside the half)
-  const int P = wmax <= 1 ? 1 : wmax <= 2 ? 2 : wmax <= 4 ? 4 : wmax <= 8 ? 8 : 16;
+  // sum of acc[k] over the half's lanes, lane k of the half ending with column k
+  const double part = transpose_reduce_p<WM, 16>(acc, lane);
+  double rhs = xo - part;
 #pragma unroll
-  for (int hh = 8; hh >= 1; hh >>= 1) {
-    if (hh < P) {   // uniform
-      const bool up = (lane & hh) != 0;
-#pragma unroll
-      for (int j = 0; j < hh; ++j) {
-        const double send = up ? acc[j] : acc[j + hh];
-        const double keep = up ? acc[j + hh] : acc[j];
-        acc[j] = keep + __shfl_xor_sync(kFull, send, hh);
-      }
-    }
-  }
-  double part = acc[0];
-  for (int m = P; m < 16; m <<= 1) part += __shfl_xor_sync(kFull, part, m);
-  double rhs = hl < ns ? ldx<CL>(xs + hl) - part : 0.0;
-  const double inv = hl < ns ? ldx<CL>(xs + rd_off + hl) : 0.0;
-  // lane k: L(i, k) for i > k, entry (i - k) of its own column
-  const double *pc = L + (hl < ns ? col_off(hl, nr) - hl : 0);
-  double lc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) lc[i] = (i > hl && i < ns) ? pc[i] : 0.0;
-#pragma unroll
-  for (int i = 15; i >= 0; --i) {
-    if (i < wmax) {   // uniform
-      if (hl == i) rhs *= inv;
-      const double zi = __shfl_sync(kFull, rhs, i, 16);
-      rhs = fma(-lc[i], zi, rhs);
-    }
+  for (int i = WM - 1; i >= 0; --i) {
+    const double zi = __shfl_sync(kFull, rhs * inv, i, 16);
+    rhs = hl == i ? zi : i > 0 ? fma(-lc[i], zi, rhs) : rhs;
   }
   if (hl < ns) xs[hl] = rhs;
   __syncwarp();
+}
+
+template <bool CL>
+__device__ void backward_half(const ISn &sn, bool valid, const double *__restrict__ Lv,
+                              const int32_t *__restrict__ rows, double *x, int64_t rd_off, int lane) {
+  const int ns = valid ? sn.ns : 0, nr = valid ? sn.ns + sn.rs : 0;
+  const double *L = Lv + (valid ? sn.lval : 0);
+  const int32_t *R = rows + (valid ? sn.rows_off : 0);
+  double *xs = x + (valid ? sn.c0 : 0);
+  const int wmax = max(ns, __shfl_xor_sync(kFull, ns, 16));
+  if (wmax <= 1) backward_half_w<CL, 1>(ns, nr, L, R, xs, x, rd_off, lane);
+  else if (wmax <= 2) backward_half_w<CL, 2>(ns, nr, L, R, xs, x, rd_off, lane);
+  else if (wmax <= 4) backward_half_w<CL, 4>(ns, nr, L, R, xs, x, rd_off, lane);
+  else if (wmax <= 8) backward_half_w<CL, 8>(ns, nr, L, R, xs, x, rd_off, lane);
+  else backward_half_w<CL, 16>(ns, nr, L, R, xs, x, rd_off, lane);
 }
 
 // One supernode by a CTA (CL = false; warps of this CTA) or by the whole
@@ -525,7 +581,9 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-__device__ void prefetch_level(const Group &g, const IPtrs &P, int lev, const double *__restrict__ Lv) {
+// descs: the descriptors too (they are in global memory)
+__device__ void prefetch_level(const Group &g, const IPtrs &P, int lev, const double *__restrict__ Lv,
+                               bool descs = true) {
   const int a = P.levptr[lev], b = P.levptr[lev + 1];
   for (int s = a + g.gw; s < b; s += g.nw) {
     const ISn sn = P.sns[s];
@@ -537,7 +595,8 @@ __device__ void prefetch_level(const Group &g, const IPtrs &P, int lev, const do
     if (g.lane == 0 && sn.rs > 0) prefetch_l2(P.rows + sn.rows_off);
   }
   // the descriptors (32 bytes each; four to a line), inside the level's range
-  for (int k = a + 4 * (32 * g.gw + g.lane); k < b; k += 4 * 32 * g.nw) prefetch_l2(P.sns + k);
+  if (descs)
+    for (int k = a + 4 * (32 * g.gw + g.lane); k < b; k += 4 * 32 * g.nw) prefetch_l2(P.sns + k);
 }
 
 // The levels [lev_lo, lev_lo + n_lev) of a subdomain by one group (CL: x
@@ -572,7 +631,7 @@ __device__ void tiny_level(const Group &g, const IPtrs &P, int a, int c, const d
     const ISn s1 = two ? P.sns[a + k + 1] : s0;
     if (s0.ns <= 16 && (!two || s1.ns <= 16)) {
       const bool hi = g.lane >= 16;
-      if (FWD) forward_half<CL>(hi ? s1 : s0, !hi || two, Lv, P.rows, x, ys, rd, g.lane);
+      if (FWD) forward_half<CL>(hi ? s1 : s0, !hi || two, Lv, P.rows, x, rd, g.lane);
       else backward_half<CL>(hi ? s1 : s0, !hi || two, Lv, P.rows, x, rd, g.lane);
     } else {
       if (FWD) forward_warp<CL>(s0, Lv, P.rows, x, ys, rd, g.lane);
@@ -816,6 +875,306 @@ __global__ void __launch_bounds__(kThreadsI, 1) implicit_kernel(const IPtrs P, c
   }
 }
 
+// ---- the tiered schedule (the default) --------------------------------------
+//
+// One CTA per subdomain leaves most of the GPU idle on a batch of fewer
+// subdomains than SMs and works through the tree's wide lower part on one
+// SM.  Here every subdomain's visited tree is cut into tiers of pieces (the
+// planner, tier_pieces): small subtrees, then the middle of the tree, then the top
+// separators.  One launch per tier and direction, one CTA per piece: forward
+// tier 0, 1, .., the top forward and backward in one, then backward down
+// the tiers.  Pieces of a tier share no rows; their updates of rows above are
+// atomic and read by later launches only, so no CTA waits for another.
+
+// q = 0, x = B^T lambda (x is zero on entry) and the reciprocal diagonals of the visited columns.
+__global__ void __launch_bounds__(256) tier_init_kernel(const IPtrs P, int per, int64_t n_dual, const double *__restrict__ Lv,
+                                                        const double *__restrict__ lam, double *__restrict__ q,
+                                                        double *__restrict__ X, uint32_t *__restrict__ status) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_dual; k += (int64_t)gridDim.x * blockDim.x)
+    q[k] = 0.0;
+  const ISub sd = P.subs[blockIdx.x / per];      // `per` CTAs to a subdomain
+  double *x = X + sd.x_off, *rd = x + P.rd_off;
+  const int gt = (int)(blockIdx.x % per * blockDim.x + threadIdx.x), nt = per * (int)blockDim.x;
+  auto recip = [&](int64_t lval, int c0, int nr, int t) {
+    bool ok;
+    const double r = pos_recip(Lv[lval + col_off(t, nr)], ok);
+    if (!ok) atomicOr(status, 1u);
+    rd[c0 + t] = ok ? r : 0.0;
+  };
+  // a warp takes 32 supernodes: a lane those of up to four columns, all lanes the columns of a wider one
+  const int lane = threadIdx.x & 31;
+  for (int s = sd.sn_lo + gt; s - lane < sd.sn_hi; s += nt) {
+    ISn sn{};
+    if (s < sd.sn_hi) sn = P.sns[s];
+    if (sn.ns <= 4) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t < sn.ns) recip(sn.lval, sn.c0, sn.ns + sn.rs, t);
+    }
+    for (uint32_t m = __ballot_sync(kFull, sn.ns > 4); m; m &= m - 1) {
+      const int k = __ffs(m) - 1, ns = __shfl_sync(kFull, sn.ns, k), rs = __shfl_sync(kFull, sn.rs, k),
+                c0 = __shfl_sync(kFull, sn.c0, k);
+      const int64_t lval = __shfl_sync(kFull, sn.lval, k);
+      for (int t = lane; t < ns; t += 32) recip(lval, c0, ns + rs, t);
+    }
+  }
+  for (int r = sd.g_lo + gt; r < sd.g_hi; r += nt) {
+    const IRow row = P.grow[r];
+    double v = 0.0;
+    for (int e = row.e_lo; e < row.e_hi; ++e) v += P.gent[e].sign * lam[P.gent[e].gj];
+    x[row.r] = v;
+  }
+}
+
+// L entries (row t0 + j, column c0 + k), j < rows, k < cols, of a panel of nr rows into dst[k][j] (stride 33:
+// a warp reads a column or a row without bank conflicts); gw / nw: the calling warp among those that copy.
+__device__ __forceinline__ void stage_block(double (*dst)[33], const double *__restrict__ L, int nr, int c0, int cols,
+                                            int t0, int rows, int gw, int nw, int lane) {
+  for (int k = gw; k < cols; k += nw)
+    if (lane < rows && t0 + lane > c0 + k) {
+      const double *src = L + col_off(c0 + k, nr) + (t0 + lane - c0 - k);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((uint32_t)__cvta_generic_to_shared(&dst[k][lane])),
+                   "l"(src)
+                   : "memory");
+    }
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// Of a group that works on one supernode of more than 32 columns: per stage the diagonal block
+// and its neighbour (forward: the rows below; backward: the columns before), the solved
+// block and the block's sums from this CTA.
+struct TierStage {
+  double D[2][32][33], N[2][32][33];
+  double ys[2][32], sum[2][32];
+};
+
+// Supernodes of more than 32 columns by a group of warps of one CTA, one barrier per 32-column block.  The chain is the triangles: the group's first
+// warp solves block b and, in the same steps, forms the next 32 rows' update (forward) or the block
+// before's sums (backward), so that its next triangle waits for nobody; meanwhile the other warps
+// update the remaining rows with the block before (forward), or sum them for the block before's
+// columns (backward), and copy the next step's blocks into shared memory.  Bound by the chain and the
+// FP64 pipe it shares: a warp alone on its SM takes a step of the chain (a multiplication and two multiply-adds
+// of 64 cycles each, two shuffles) in 241 cycles, one beside 15 others with multiply-adds in 1495.  588
+// columns: 128 us forward, 143 backward (a cluster of eight SMs whose first has the chain to itself:
+// 106 and 147, and slower on the levels below).
+__device__ void forward_big(const Group &g, const ISn &sn, const double *__restrict__ Lv,
+                            const int32_t *__restrict__ rows, double *x, int64_t rd_off, TierStage &st) {
+  const int ns = sn.ns, nr = ns + sn.rs, nb = (ns + 31) >> 5, lane = g.lane;
+  const double *L = Lv + sn.lval;
+  const int32_t *R = rows + sn.rows_off;
+  double *xs = x + sn.c0;
+  auto stage = [&](int b, int gw, int nw) {
+    const int w = min(32, ns - 32 * b);
+    stage_block(st.D[b & 1], L, nr, 32 * b, w, 32 * b, w, gw, nw, lane);
+    if (b + 1 < nb) stage_block(st.N[b & 1], L, nr, 32 * b, 32, 32 * b + 32, min(32, nr - 32 * b - 32), gw, nw, lane);
+  };
+  g.sync_cta();                       // the group's stages are free
+  stage(0, g.gw, g.nw);
+  stage_wait();
+  g.sync_cta();
+  double accn = 0.0;                  // the first warp's: update of rows 32 b + lane by block b - 1
+  for (int b = 0; b < nb; ++b) {
+    const int w = min(32, ns - 32 * b);
+    if (g.gw == 0) {
+      const bool own = lane < w;
+      const double inv = own ? xs[rd_off + 32 * b + lane] : 0.0;
+      double xi = own ? xs[32 * b + lane] - accn : 0.0;
+      const int t = 32 * b + lane;
+      if (b > 0 && !own && t < nr) atomicAdd(x + R[t - ns], -accn);
+      const double(*D)[33] = st.D[b & 1], (*N)[33] = st.N[b & 1];
+      const bool nrow = b + 1 < nb && t + 32 < nr;
+      accn = 0.0;
+#pragma unroll 8
+      for (int k = 0; k < w; ++k) {
+        const double l = lane > k ? D[k][lane] : 0.0, n = nrow ? N[k][lane] : 0.0;
+        const double yk = __shfl_sync(kFull, xi, k) * __shfl_sync(kFull, inv, k);
+        xi = lane == k ? yk : fma(-l, yk, xi);
+        accn = fma(n, yk, accn);
+      }
+      if (own) xs[32 * b + lane] = xi;
+      st.ys[b & 1][lane] = own ? xi : 0.0;
+    } else {
+      if (b + 1 < nb) stage(b + 1, g.gw - 1, g.nw - 1);
+      if (b > 0)
+        for (int t0 = 32 * (b + g.gw); t0 < nr; t0 += 32 * (g.nw - 1))
+          forward_panel_chunk<false>(L, R, ns, nr, 32 * (b - 1), 32, t0, st.ys[(b - 1) & 1], xs, x, lane);
+      stage_wait();
+    }
+    g.sync_cta();
+  }
+  const int kb = 32 * (nb - 1);
+  for (int t0 = ns + 32 * g.gw; t0 < nr; t0 += 32 * g.nw)
+    forward_panel_chunk<false>(L, R, ns, nr, kb, ns - kb, t0, st.ys[(nb - 1) & 1], xs, x, lane);
+}
+
+// red: one 32-double row per warp of the CTA
+__device__ void backward_big(const Group &g, const ISn &sn, const double *__restrict__ Lv,
+                             const int32_t *__restrict__ rows, double *x, int64_t rd_off, TierStage &st,
+                             double (*red)[32]) {
+  const int ns = sn.ns, nr = ns + sn.rs, nb = (ns + 31) >> 5, lane = g.lane;
+  const double *L = Lv + sn.lval;
+  const int32_t *R = rows + sn.rows_off;
+  double *xs = x + sn.c0;
+  // step b: the triangle of block b, and the rows of block b under the columns of block b - 1
+  auto stage = [&](int b, int gw, int nw) {
+    const int w = min(32, ns - 32 * b);
+    stage_block(st.D[b & 1], L, nr, 32 * b, w, 32 * b, w, gw, nw, lane);
+    if (b > 0) stage_block(st.N[b & 1], L, nr, 32 * (b - 1), 32, 32 * b, w, gw, nw, lane);
+  };
+  // st.sum[b & 1] = the sums over rows t_lo, .. of L(t, column) z_t for block b's columns; the
+  // 32-row chunks are shared by the group's warps from first_warp on
+  auto sums = [&](int b, int t_lo, int first_warp) {
+    const int kb = 32 * b, w = min(32, ns - kb), idx = g.gw - first_warp, cnt = g.nw - first_warp;
+    if (t_lo + 32 * idx < nr) {
+      double acc[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) acc[k] = 0.0;
+      for (int t0 = t_lo + 32 * idx; t0 < nr; t0 += 32 * cnt)
+        backward_panel_chunk<false>(L, R, ns, nr, kb, w, t0, xs, x, acc, lane);
+      red[g.warp][lane] = transpose_reduce_w(acc, lane, w);
+    }
+    asm volatile("bar.sync %0, %1;\n" ::"r"(8 + g.slot), "r"(32 * cnt) : "memory");
+    if (idx == 0) {
+      const int have = min(cnt, (nr - t_lo + 31) >> 5);
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int v = 0; v < have; v += 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (v + j < have) s[j] += red[g.warp + v + j][lane];
+      st.sum[b & 1][lane] = (s[0] + s[1]) + (s[2] + s[3]);
+    }
+  };
+  g.sync_cta();
+  stage(nb - 1, g.gw, g.nw);
+  sums(nb - 1, ns, 0);
+  stage_wait();
+  g.sync_cta();
+  double accp = 0.0;
+  for (int b = nb - 1; b >= 0; --b) {
+    const int w = min(32, ns - 32 * b);
+    if (g.gw == 0) {
+      const bool own = lane < w;
+      const double inv = own ? xs[rd_off + 32 * b + lane] : 0.0;
+      const double part = accp + st.sum[b & 1][lane];
+      double rhs = own ? xs[32 * b + lane] - part : 0.0;
+      const double(*D)[33] = st.D[b & 1], (*N)[33] = st.N[b & 1];
+      accp = 0.0;
+#pragma unroll 8
+      for (int i = w - 1; i >= 0; --i) {
+        const double l = lane < i ? D[lane][i] : 0.0, n = b > 0 ? N[lane][i] : 0.0;
+        const double zi = __shfl_sync(kFull, rhs * inv, i);
+        rhs = lane == i ? zi : fma(-l, zi, rhs);
+        accp = fma(n, zi, accp);
+      }
+      if (own) xs[32 * b + lane] = rhs;
+    } else if (b > 0) {
+      stage(b - 1, g.gw - 1, g.nw - 1);
+      sums(b - 1, 32 * b + w, 1);
+      stage_wait();
+    }
+    g.sync_cta();
+  }
+}
+
+constexpr int kTierSns = 768;     // supernode descriptors kept in shared memory (of a piece's; the rest are read from global)
+constexpr int kTierLevs = 63;
+constexpr int kTinyWork = 512;    // entries of a supernode up to which half a warp takes it
+
+template <int kGroups>            // groups that can work on supernodes of more than 32 columns side by side
+struct TierShared {
+  TierStage stage[kGroups];
+  double red[kWarps][32];
+  double ys[kWarps][32];
+  double red_cta[kWarps * 32];
+  ISn sns[kTierSns];
+  int32_t levptr[kTierLevs + 1];
+  int take_ctr;
+};
+
+// One level of a piece: supernodes [a, a + c), largest first.
+template <bool kForward, int kGroups>
+__device__ __forceinline__ void tier_level(const Group &g, const IPtrs &P, int a, int c, const double *__restrict__ Lv,
+                                           double *x, TierShared<kGroups> &sm, int &base) {
+  const int W = nwarps(), warp = g.warp, lane = g.lane;
+  const int64_t rd = P.rd_off;
+  const ISn s0 = P.sns[a];
+  const bool tiny = s0.ns * (s0.ns + 1) / 2 + s0.ns * s0.rs <= kTinyWork;
+  if (tiny || 2 * c >= W) {
+    // a warp or half a warp per supernode
+    if (tiny || s0.ns <= 16) {
+      tiny_level<false, kForward>(g, P, a, c, Lv, x, sm.ys[warp], rd, &sm.take_ctr, base);
+    } else {
+      for (int k = take(&sm.take_ctr, base, lane); k < c; k = take(&sm.take_ctr, base, lane)) {
+        if (kForward) forward_warp<false>(P.sns[a + k], Lv, P.rows, x, sm.ys[warp], rd, lane);
+        else backward_warp<false>(P.sns[a + k], Lv, P.rows, x, rd, lane);
+      }
+      base += c + W;
+    }
+  } else {
+    // every supernode on a group of the warps, kGroups side by side where one has more than 32 columns
+    bool wide = false;
+    for (int s = 0; s < c; ++s) wide = wide || P.sns[a + s].ns > 32;
+    const int at_once = wide ? min(c, kGroups) : c;
+    const int j = warp * at_once / W, w0 = (W * j + at_once - 1) / at_once, nw = (W * (j + 1) + at_once - 1) / at_once - w0;
+    const Group sg = sub_group(warp, lane, w0, nw, j);
+    for (int s = j; s < c; s += at_once) {
+      const ISn sn = P.sns[a + s];
+      if (sn.ns > 32 && nw > 1) {
+        if (kForward) forward_big(sg, sn, Lv, P.rows, x, rd, sm.stage[j]);
+        else backward_big(sg, sn, Lv, P.rows, x, rd, sm.stage[j], sm.red);
+      } else {
+        if (kForward) forward_group<false>(sg, sn, Lv, P.rows, x, sm.ys[warp], rd);
+        else backward_group<false>(sg, sn, Lv, P.rows, x, rd, &sm.red[0][0], sm.red_cta);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+template <bool kForward, bool kBackward, int kGroups>
+__global__ void __launch_bounds__(kThreadsI, 1) tier_kernel(IPtrs P, int first, const double *__restrict__ Lv,
+                                                            double *q, double *X) {
+  extern __shared__ __align__(16) unsigned char tier_smem[];
+  TierShared<kGroups> &sm = *reinterpret_cast<TierShared<kGroups> *>(tier_smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Group g = cta_group(warp, lane);
+  const IPiece pc = P.pieces[first + blockIdx.x];
+  double *x = X + P.subs[pc.sub].x_off;
+  if (threadIdx.x == 0) sm.take_ctr = 0;
+  // the piece's levels and descriptors, so that a level starts without dependent global loads
+  const int s_lo = P.levptr[pc.lev_lo], s_hi = P.levptr[pc.lev_lo + pc.n_lev];
+  if (pc.n_lev <= kTierLevs) {
+    for (int k = threadIdx.x; k <= pc.n_lev; k += blockDim.x) sm.levptr[k] = P.levptr[pc.lev_lo + k];
+  }
+  const bool in_smem = s_hi - s_lo <= kTierSns;
+  if (in_smem) {
+    const int4 *src = reinterpret_cast<const int4 *>(P.sns + s_lo);
+    int4 *dst = reinterpret_cast<int4 *>(sm.sns);
+    for (int k = threadIdx.x; k < 2 * (s_hi - s_lo); k += blockDim.x) dst[k] = src[k];
+    P.sns = sm.sns - s_lo;
+  }
+  if (pc.n_lev <= kTierLevs) P.levptr = sm.levptr - pc.lev_lo;
+  __syncthreads();
+  int base = 0;
+  if (kForward) {
+    prefetch_level(g, P, pc.lev_lo, Lv, !in_smem);
+    for (int l = 0; l < pc.n_lev; ++l) {
+      if (l + 1 < pc.n_lev) prefetch_level(g, P, pc.lev_lo + l + 1, Lv, !in_smem);
+      const int a = P.levptr[pc.lev_lo + l], b = P.levptr[pc.lev_lo + l + 1];
+      tier_level<true, kGroups>(g, P, a, b - a, Lv, x, sm, base);
+    }
+  }
+  if (kBackward) {
+    if (!kForward) prefetch_level(g, P, pc.lev_lo + pc.n_lev - 1, Lv, !in_smem);
+    for (int l = pc.n_lev - 1; l >= 0; --l) {
+      if (l > 0) prefetch_level(g, P, pc.lev_lo + l - 1, Lv, !in_smem);
+      const int a = P.levptr[pc.lev_lo + l], b = P.levptr[pc.lev_lo + l + 1];
+      tier_level<false, kGroups>(g, P, a, b - a, Lv, x, sm, base);
+    }
+    scatter_q<false>(P, pc.s_lo, pc.s_hi, x, q, (int)threadIdx.x, (int)blockDim.x);
+  }
+}
+
 }  // namespace
 
 struct sci_ctx {
@@ -831,6 +1190,8 @@ struct sci_ctx {
   int64_t n_pair_subdomains = 0;    // subdomains on CTA pairs (the launch then needs clusters)
   int64_t x_total = 0;              // doubles of all subdomains' x (the reciprocal diagonals follow)
   int32_t warps = kWarps;           // warps per CTA of the launch
+  bool tiered = false;              // the tiered schedule: no cluster or pair was asked for
+  int32_t tier_first[kTiers + 1] = {};   // pieces of tier t: [tier_first[t], tier_first[t + 1])
 
   IPtrs ptrs() const {
     const uint8_t *b = static_cast<const uint8_t *>(plan_dev);
@@ -843,6 +1204,7 @@ struct sci_ctx {
     p.gent = reinterpret_cast<const IEnt *>(b + hdr.sec_off[5]);
     p.sent = reinterpret_cast<const ISEnt *>(b + hdr.sec_off[6]);
     p.items = reinterpret_cast<const IItem *>(b + hdr.sec_off[7]);
+    p.pieces = reinterpret_cast<const IPiece *>(b + hdr.piece_off);
     p.rd_off = x_total;
     return p;
   }
@@ -912,6 +1274,42 @@ bool split_tree(const sc::SubPlan &S, const std::vector<int32_t> &vis, std::vect
   return false;
 }
 
+// Tier and piece (numbered within the tier) of every visited supernode of one subdomain.  Tier t: of
+// what the tiers before left, the maximal subtrees of at most cap[t] entries of L (cap 0: none); the last
+// tier: the rest, one piece.  Small subtrees share a piece up to the cap.
+void tier_pieces(const sc::SubPlan &S, const std::vector<int32_t> &vis, const int64_t (&cap)[kTiers - 1],
+                 std::vector<int8_t> &tier, std::vector<int32_t> &piece) {
+  const int32_t nsn = (int32_t)S.sn_c0.size();
+  tier.assign(nsn, kTiers - 1);
+  piece.assign(nsn, 0);
+  for (int t = 0; t < kTiers - 1; ++t) {
+    if (cap[t] <= 0) continue;
+    std::vector<int64_t> w(nsn, 0);
+    for (int32_t s : vis) {                       // children before parents
+      if (tier[s] < t) continue;
+      w[s] += (int64_t)S.sn_ns[s] * (S.sn_ns[s] + 1) / 2 + (int64_t)S.sn_ns[s] * S.sn_rs[s];
+      if (S.sparent[s] >= 0) w[S.sparent[s]] += w[s];
+    }
+    int32_t cur = 0;
+    int64_t load = 0;
+    for (auto it = vis.rbegin(); it != vis.rend(); ++it) {        // parents before children
+      const int32_t s = *it, p = S.sparent[s];
+      if (tier[s] < t || w[s] > cap[t]) continue;
+      tier[s] = (int8_t)t;
+      if (p >= 0 && tier[p] == t) {
+        piece[s] = piece[p];
+      } else {                                    // the root of a subtree
+        if (load > 0 && load + w[s] > cap[t]) {
+          ++cur;
+          load = 0;
+        }
+        load += w[s];
+        piece[s] = cur;
+      }
+    }
+  }
+}
+
 sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t cluster_min_work,
                 int32_t pairs) {
   for (int32_t i = 0; i < nsub; ++i)
@@ -949,10 +1347,24 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return work[a] > work[b]; });
   if (cluster_min_work < 0)
     cluster_min_work = std::max<int64_t>(1, 2 * nnz_all / std::max<int64_t>(1, std::min<int64_t>(kCtaSlots, nsub)) + 1);
+  if (ctx->tiered) cluster_min_work = std::numeric_limits<int64_t>::max();   // no clusters
   // CTA pairs only on request: measured on GB300 (config 2, 64 subdomains on
   // 152 SMs) a pair took 2.51 ms against 2.20 ms for one CTA per subdomain --
   // the subtrees are not the critical path, the per-level chains are
   const bool want_pairs = pairs == 1;
+  // The tiers' caps: halves of the largest subdomain's entries (a nested-dissection tree halves its
+  // subtrees level by level), not below a quarter of an SM's share of the batch nor 4000 entries, which a
+  // CTA works through in about the time of a launch.  GB300, us with 1 / 2 / 3 / 4 / 5 tiers: 64 heat cubes
+  // 1130 / 758 / 772 / 807 / 900, 8 elasticity cubes and 16 squares 2055 / 1502 / 1564 / 1314 / 1563, four elasticity
+  // cubes 1640 / 1620 / 1407 / 1414 / 1111, 36 squares 430 / 475 / 294 / 314 / 322.
+  int64_t cap[kTiers - 1] = {};
+  if (ctx->tiered && nsub > 0) {
+    const double least = std::max((double)nnz_all / (4 * kCtaSlots), 4000.0);
+    double w = (double)work[order[0]];
+    for (int t = kTiers - 2; t >= 0 && (w *= 0.5) >= least; --t) cap[t] = (int64_t)w;
+  }
+  std::vector<IPiece> pieces[kTiers];
+  std::vector<int64_t> piece_work[kTiers];
   std::vector<int8_t> is_pair(nsub, 0);
   for (int32_t i : order) {
     const sc::SubPlan &S = P[i];
@@ -967,6 +1379,8 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
     std::vector<int8_t> part;
     const bool pair = want_pairs && work[i] < cluster_min_work && split_tree(S, vis, part);
     if (!pair) part.assign(nsn, 2);
+    std::vector<int32_t> piece(nsn, 0);
+    if (ctx->tiered) tier_pieces(S, vis, cap, part, piece);
     is_pair[i] = pair;
     // (part, level, work descending): parts A, B, then the top, one level
     // sequence each; within a level the largest supernodes first, so that the
@@ -974,6 +1388,7 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
     auto snw = [&](int32_t s) { return (int64_t)S.sn_ns[s] * (S.sn_ns[s] + 1) / 2 + (int64_t)S.sn_ns[s] * S.sn_rs[s]; };
     std::stable_sort(vis.begin(), vis.end(), [&](int32_t a, int32_t b) {
       if (part[a] != part[b]) return part[a] < part[b];
+      if (piece[a] != piece[b]) return piece[a] < piece[b];
       if (h[a] != h[b]) return h[a] < h[b];
       return snw(a) > snw(b);
     });
@@ -982,15 +1397,27 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
     sd.n = D.n;
     sd.sn_lo = (int32_t)sns.size();
     sd.lev_lo = (int32_t)levptr.size();
-    int32_t cur_part = -1, cur_h = -1, nlev = 0, nlev_part[3] = {0, 0, 0};
+    int32_t cur_part = -1, cur_piece = -1, cur_h = -1, nlev = 0, nlev_part[kTiers] = {}, deepest = 0;
     for (int32_t s : vis) {
-      if (part[s] != cur_part || h[s] != cur_h) {   // a new level (heights are increasing within a part)
+      const bool new_piece = part[s] != cur_part || piece[s] != cur_piece;
+      if (new_piece && ctx->tiered) {
+        IPiece pc{};
+        pc.sub = (int32_t)subs.size();
+        pc.lev_lo = (int32_t)levptr.size();
+        pieces[part[s]].push_back(pc);
+        piece_work[part[s]].push_back(0);
+      }
+      if (new_piece || h[s] != cur_h) {   // a new level (heights are increasing within a part's piece)
         levptr.push_back((int32_t)sns.size());
         cur_part = part[s];
+        cur_piece = piece[s];
         cur_h = h[s];
         ++nlev;
         ++nlev_part[cur_part];
+        if (ctx->tiered) ++pieces[cur_part].back().n_lev;
       }
+      deepest = std::max(deepest, h[s] + 1);
+      if (ctx->tiered) piece_work[cur_part].back() += snw(s);
       ISn sn{};
       const int32_t c0 = S.sn_c0[s], ns = S.sn_ns[s], rs = S.sn_rs[s];
       // the kernel addresses a panel with 32-bit offsets
@@ -1009,13 +1436,13 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
     }
     sd.sn_hi = (int32_t)sns.size();
     sd.n_lev = nlev;
-    sd.n_lev_a = nlev_part[0];
-    sd.n_lev_b = nlev_part[1];
+    sd.n_lev_a = pair ? nlev_part[0] : 0;
+    sd.n_lev_b = pair ? nlev_part[1] : 0;
     levptr.push_back(sd.sn_hi);
-    max_lev = std::max<int64_t>(max_lev, sd.n_lev);
+    max_lev = std::max<int64_t>(max_lev, ctx->tiered ? deepest : sd.n_lev);
     // B^T by row (gather) and by entry (scatter)
     std::vector<std::pair<int32_t, int32_t>> ent;   // (row, entry index)
-    std::vector<ISEnt> by_part[3];                    // scatter entries by the part of their row
+    std::vector<ISEnt> by_part[kTiers];               // scatter entries by the part of their row
     for (int32_t j = 0; j < D.m; ++j)
       for (int32_t e = D.Bt_colptr[j]; e < D.Bt_colptr[j + 1]; ++e) {
         ent.emplace_back(D.Bt_rowind[e], e);
@@ -1023,11 +1450,31 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
         by_part[part[S.snode_of[r]]].push_back(ISEnt{r, D.lambda_map[j], (int32_t)D.Bt_sign[e], 0});
       }
     sd.s_lo = (int32_t)sent.size();
-    sent.insert(sent.end(), by_part[0].begin(), by_part[0].end());
-    sd.s_mid1 = (int32_t)sent.size();
-    sent.insert(sent.end(), by_part[1].begin(), by_part[1].end());
-    sd.s_mid2 = (int32_t)sent.size();
-    sent.insert(sent.end(), by_part[2].begin(), by_part[2].end());
+    if (ctx->tiered) {                              // by the piece of their row
+      for (auto &all : by_part)
+        std::stable_sort(all.begin(), all.end(), [&](const ISEnt &x, const ISEnt &y) {
+          return piece[S.snode_of[x.r]] < piece[S.snode_of[y.r]];
+        });
+      for (int t = 0; t < kTiers; ++t) {
+        // this subdomain's pieces of the tier are the last ones, numbered upwards from 0
+        size_t k = pieces[t].size();
+        while (k > 0 && pieces[t][k - 1].sub == (int32_t)subs.size()) --k;
+        size_t e = 0;
+        for (int32_t num = 0; k < pieces[t].size(); ++k, ++num) {
+          pieces[t][k].s_lo = (int32_t)(sent.size() + e);
+          while (e < by_part[t].size() && piece[S.snode_of[by_part[t][e].r]] == num) ++e;
+          pieces[t][k].s_hi = (int32_t)(sent.size() + e);
+        }
+        sent.insert(sent.end(), by_part[t].begin(), by_part[t].end());
+      }
+      sd.s_mid1 = sd.s_mid2 = sd.s_lo;
+    } else {
+      sent.insert(sent.end(), by_part[0].begin(), by_part[0].end());
+      sd.s_mid1 = (int32_t)sent.size();
+      sent.insert(sent.end(), by_part[1].begin(), by_part[1].end());
+      sd.s_mid2 = (int32_t)sent.size();
+      sent.insert(sent.end(), by_part[2].begin(), by_part[2].end());
+    }
     std::vector<int32_t> col_of(ent.size());
     for (int32_t j = 0; j < D.m; ++j)
       for (int32_t e = D.Bt_colptr[j]; e < D.Bt_colptr[j + 1]; ++e) col_of[e] = j;
@@ -1109,6 +1556,17 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
   H.sec_off[5] = put_section(blob, gent);
   H.sec_off[6] = put_section(blob, sent);
   H.sec_off[7] = put_section(blob, items);
+  std::vector<IPiece> all_pieces;
+  for (int t = 0; t < kTiers; ++t) {
+    std::vector<int32_t> o(pieces[t].size());
+    std::iota(o.begin(), o.end(), 0);
+    std::stable_sort(o.begin(), o.end(), [&](int32_t a, int32_t b) { return piece_work[t][a] > piece_work[t][b]; });
+    ctx->tier_first[t] = (int32_t)all_pieces.size();
+    for (int32_t k : o) all_pieces.push_back(pieces[t][k]);
+  }
+  ctx->tier_first[kTiers] = (int32_t)all_pieces.size();
+  H.n_pieces = (int64_t)all_pieces.size();
+  H.piece_off = put_section(blob, all_pieces);
   blob.resize((blob.size() + 255) & ~size_t(255));
   std::memcpy(blob.data(), &H, sizeof(H));
   sci_sizes &z = ctx->sizes;
@@ -1123,6 +1581,42 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
   z.flops = 4.0 * (double)nnz_all;
   z.n_cluster_subdomains = n_big;
   z.bytes = 16.0 * (double)nnz_all + 16.0 * (double)m_all;
+  return SC_OK;
+}
+
+sc_status apply_tiered(sci_ctx *ctx, const double *Lv, const double *lam, double *q, double *X, uint32_t *status,
+                       cudaStream_t st) {
+  // the status word and every x (they follow it in the workspace)
+  cudaError_t e = cudaMemsetAsync(status, 0, 256 + sizeof(double) * (size_t)ctx->x_total, st);
+  if (e == cudaSuccess && ctx->nsub > 0) {
+    const IPtrs P = ctx->ptrs();
+    const int per = (int)std::max<int64_t>(1, std::min<int64_t>(16, 8 * kCtaSlots / ctx->nsub));
+    tier_init_kernel<<<(unsigned)per * (unsigned)ctx->nsub, 256, 0, st>>>(P, per, ctx->n_dual, Lv, lam, q, X, status);
+    for (int k = 0; k < 2 * kTiers - 1 && e == cudaSuccess; ++k) {
+      const int t = k < kTiers ? k : 2 * kTiers - 2 - k;
+      const unsigned n = (unsigned)(ctx->tier_first[t + 1] - ctx->tier_first[t]);
+      if (n == 0) continue;
+      // a tier with more pieces than SMs: 8 warps and two CTAs per SM
+      const bool two = n > (unsigned)kCtaSlots;
+      const unsigned nt = two ? kThreadsI / 2 : kThreadsI;
+      auto launch = [&](auto kernel, size_t smem) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) kernel<<<n, nt, smem, st>>>(P, (int)ctx->tier_first[t], Lv, q, X);
+      };
+      const bool up = k < kTiers - 1, down = k > kTiers - 1;
+#define SCI_TIER(G)                                                      \
+  if (up) launch(tier_kernel<true, false, G>, sizeof(TierShared<G>));     \
+  else if (down) launch(tier_kernel<false, true, G>, sizeof(TierShared<G>)); \
+  else launch(tier_kernel<true, true, G>, sizeof(TierShared<G>));
+      if (two) { SCI_TIER(2) }
+      else { SCI_TIER(4) }
+#undef SCI_TIER
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
+  } else if (e == cudaSuccess && ctx->n_dual > 0) {
+    e = cudaMemsetAsync(q, 0, sizeof(double) * (size_t)ctx->n_dual, st);
+  }
+  if (e != cudaSuccess) return ifail(ctx, SC_ERR_CUDA, std::string("sci_apply: ") + cudaGetErrorString(e));
   return SC_OK;
 }
 
@@ -1143,6 +1637,7 @@ sc_status sci_plan(sci_ctx **out, int32_t nsub, const sc_subdomain_desc *subdoma
   ctx->n_dual = n_dual;
   try {
     if (opt && (opt->pairs < -1 || opt->pairs > 1)) return ifail(ctx, SC_ERR_INVALID_ARG, "pairs must be -1, 0 or 1");
+    ctx->tiered = !opt || (opt->cluster_min_work < 0 && opt->pairs != 1);
     return build(ctx, nsub, subdomains, opt ? opt->cluster_min_work : -1, opt ? opt->pairs : 0);
   } catch (const std::bad_alloc &) {
     return ifail(ctx, SC_ERR_OOM, "host allocation failed while planning");
@@ -1183,6 +1678,7 @@ sc_status sci_apply(sci_ctx *ctx, const double *L_values_dev, const double *lamb
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint32_t *status = static_cast<uint32_t *>(ws_dev);
   double *X = reinterpret_cast<double *>(static_cast<uint8_t *>(ws_dev) + 256);
+  if (ctx->tiered) return apply_tiered(ctx, L_values_dev, lambda_dev, q_dev, X, status, st);
   cudaError_t e = cudaMemsetAsync(status, 0, sizeof(uint32_t), st);
   if (e == cudaSuccess && ctx->n_dual > 0) e = cudaMemsetAsync(q_dev, 0, sizeof(double) * (size_t)ctx->n_dual, st);
   if (e == cudaSuccess && ctx->n_items > 0) {
