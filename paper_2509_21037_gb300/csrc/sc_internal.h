@@ -178,7 +178,8 @@ struct sc_ctx {
   // per wave, launch groups by variant (index 0 = FP64, 3..7 = digits): first item, count
   struct WaveGroups {
     int64_t trsm[sc::kNumVariants][2] = {}, syrk[sc::kNumVariants][2] = {}, sblk[sc::kNumVariants][2] = {};
-    int trsm_cols = 16, syrk_ctas = 1;   // FP64 group: columns per TRSM warp, CTAs per SYRK task (sc_plan.cpp)
+    // by variant: columns per TRSM warp (sc_plan.cpp); FP64 group: CTAs per SYRK task
+    int trsm_cols[sc::kNumVariants] = {}, syrk_ctas = 1;
   };
   std::vector<WaveGroups> waves;
   std::vector<int32_t> sub_wave;     // wave of every subdomain
@@ -225,7 +226,7 @@ int launch_groups(sc_ctx &c, int w, const double *Lv, const double *invd, void *
                   void *stream, bool aux);
 // split-precision launchers: one variant group of one wave (S digits, items [base, base + count))
 int launch_lpack_split(const sc_ctx &c, int S, int64_t base, int64_t count, const double *Lv, void *ws, void *stream);
-int launch_trsm_split(const sc_ctx &c, int S, int64_t base, int64_t count, const double *Lv, const double *invd,
+int launch_trsm_split(const sc_ctx &c, int S, int cols, int64_t base, int64_t count, const double *Lv, const double *invd,
                       void *ws, double *Y, void *stream);
 int launch_colexp_reset(const sc_ctx &c, void *ws, void *stream);
 // balanced: digits in [-128, 128] against twice the column bound (the tcgen05 SYRK's planes)

@@ -541,17 +541,19 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       g[1]++;
     }
   };
-  // total and longest cost of every wave's FP64 group
+  // total and longest cost of every wave's groups
   auto each_group = [&](const std::vector<double> &cost, const std::vector<int8_t> &var,
                         const std::vector<int32_t> &wave, const std::vector<int32_t> &o, auto set) {
-    std::vector<double> total(ctx->waves.size(), 0.0), longest(ctx->waves.size(), 0.0);
+    struct Sum { double total[kNumVariants] = {}, longest[kNumVariants] = {}; };
+    std::vector<Sum> sum(ctx->waves.size());
     for (int32_t k : o) {
-      if (var[k] != 0) continue;
-      total[wave[k]] += cost[k];
-      longest[wave[k]] = std::max(longest[wave[k]], cost[k]);
+      Sum &s = sum[wave[k]];
+      s.total[var[k]] += cost[k];
+      s.longest[var[k]] = std::max(s.longest[var[k]], cost[k]);
     }
-    for (size_t w = 0; w < total.size(); ++w)
-      if (total[w] > 0.0) set(ctx->waves[w], total[w], longest[w]);
+    for (size_t w = 0; w < sum.size(); ++w)
+      for (int v = 0; v < kNumVariants; ++v)
+        if (sum[w].total[v] > 0.0) set(ctx->waves[w], v, sum[w].total[v], sum[w].longest[v]);
   };
   {
     auto o = order_by(trsm_cost, trsm_var, trsm_wave);
@@ -575,9 +577,12 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
     // columns: 64 heat cubes 22.9 / 19.8 / 18.4 / 17.9 / 17.4 (rule: 16), 8 elasticity cubes
     // 7.80 / 7.78 / 10.7 / 15.3 / 33.7 (2), 36 plane squares 0.355 / 0.280 / 0.299 / 0.425 / 0.82 (2),
     // one square 0.031 / 0.035 / 0.050 / 0.065 / 0.10 (1).
-    each_group(trsm_cost, trsm_var, trsm_wave, o, [&](sc_ctx::WaveGroups &g, double total, double longest) {
-      g.trsm_cols = 16;
-      while (g.trsm_cols > 1 && longest * g.trsm_cols / kChunk > 0.5 * total / (4 * kGridSMs)) g.trsm_cols /= 2;
+    // The split-precision TRSM takes 2 or 4 columns per warp by the same rule (7 digits, ms at 2 / 4: 64 heat cubes
+    // 7.7 / 6.3 (rule: 4), 27 small ones 0.37 / 0.30 (4), 8 elasticity cubes 2.3 / 2.9 (2), 36 squares 0.32 / 0.39 (2)).
+    each_group(trsm_cost, trsm_var, trsm_wave, o, [&](sc_ctx::WaveGroups &g, int v, double total, double longest) {
+      int &cols = g.trsm_cols[v];
+      cols = v == 0 ? 16 : 4;
+      while (cols > (v == 0 ? 1 : 2) && longest * cols / kChunk > 0.5 * total / (4 * kGridSMs)) cols /= 2;
     });
     std::vector<TrsmTask> t2(trsm.size());
     for (size_t k = 0; k < o.size(); ++k) t2[k] = trsm[o[k]];
@@ -590,7 +595,8 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
     // most a quarter of an SM's share of the whole, else 4 or 8.  GB300, ms at 1 / 4 / 8: 64 heat cubes
     // 30.3 / 30.7 / 31.3 (rule: 1), 8 elasticity cubes 6.46 / 6.49 / 6.57 (1), 36 plane squares
     // 0.196 / 0.153 / 0.155 (4), one square 0.031 / 0.018 / 0.014 (8).
-    each_group(syrk_cost, syrk_var, syrk_wave, o, [&](sc_ctx::WaveGroups &g, double total, double longest) {
+    each_group(syrk_cost, syrk_var, syrk_wave, o, [&](sc_ctx::WaveGroups &g, int v, double total, double longest) {
+      if (v != 0) return;
       const double r = longest * kGridSMs / total;
       g.syrk_ctas = r <= 0.25 ? 1 : r <= 1.0 ? 4 : 8;
     });

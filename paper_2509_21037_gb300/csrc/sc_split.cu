@@ -25,7 +25,7 @@
 //     FP64 and one scaling (the FP64 pipe is the scarce resource on GB300).
 //
 // L and Y are cut into digit planes once per assembly (lpack_kernel after
-// the reciprocal diagonal; ycolexp/yslice after the TRSM), so the TRSM and
+// the reciprocal diagonal; yslice after the TRSM, which leaves Y's column bounds), so the TRSM and
 // SYRK tasks only load BF16 planes.
 //
 // Only pairs with t + t' <= S - 1 are formed (S(S+1)/2 products); the terms
@@ -38,12 +38,17 @@
 
 #include "sc_digits.cuh"
 #include "sc_internal.h"
+#include "sc_trsm.cuh"
 
 namespace sc {
 
 namespace {
 
 using namespace digits;
+
+// TRSM blocks of at most kDirect columns update the rows below in FP64, a multiply-add per
+// column and entry of Y against the two operations that an entry costs after the digit products.
+constexpr int kDirect = 4;
 
 constexpr int kPad = 40;   // bf16 row stride of a digit plane (conflict-free fragment loads)
 
@@ -59,10 +64,10 @@ __device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16 *p) {
   return *reinterpret_cast<const uint32_t *>(p);
 }
 
-
 // Digit planes of L's panel rows below one 32x32 diagonal block (one CTA per
 // (supernode, block) item; one thread per panel row, so every CSC column is
-// read contiguously).
+// read contiguously).  The 16 words of a plane's row are stored word w at 4 (w mod 4) + w / 4: the four that a lane
+// of the update needs are then one 16-byte load.  Blocks of up to kDirect columns need no planes.
 template <int S>
 __global__ void __launch_bounds__(kThreads) lpack_kernel(const PlanPtrs P, const double *__restrict__ Lv,
                                                          __nv_bfloat16 *__restrict__ Ld,
@@ -73,6 +78,7 @@ __global__ void __launch_bounds__(kThreads) lpack_kernel(const PlanPtrs P, const
   const int nrow = s.ns + s.rs;
   const int kb = 32 * b, kw = min(32, s.ns - kb);
   const int nb = nrow - kb - kw;
+  if (kw <= kDirect) return;
   const int64_t base = s.ld_off + (int64_t)b * nrow - 16LL * b * (b + 1);
   for (int r = threadIdx.x; r < nb; r += kThreads) {
     const int p = kb + kw + r;
@@ -100,7 +106,7 @@ __global__ void __launch_bounds__(kThreads) lpack_kernel(const PlanPtrs P, const
         uint32_t w[4];
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-          const int q = 8 * g + 2 * h;
+          const int q = 2 * (4 * h + g);          // word 4 h + g of the row
           const __nv_bfloat16 lo = digit_bf16(X[q], d, (neg >> q) & 1u);
           const __nv_bfloat16 hi = digit_bf16(X[q + 1], d, (neg >> (q + 1)) & 1u);
           w[h] = (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
@@ -108,21 +114,6 @@ __global__ void __launch_bounds__(kThreads) lpack_kernel(const PlanPtrs P, const
         row[g] = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
-  }
-}
-
-// Column exponent bounds of Y over one (supernode, 32-row block) item.
-__global__ void __launch_bounds__(kThreads) ycolexp_kernel(const PlanPtrs P, const double *__restrict__ Y,
-                                                           int *__restrict__ colexp) {
-  const int si = P.sblk[2 * blockIdx.x], b = P.sblk[2 * blockIdx.x + 1];
-  const SnDev s = P.sns[si];
-  const SubDev sd = P.subs[s.sub];
-  const int ws = s.jhi - s.jlo;
-  const int r0 = 32 * b, r1 = min(s.ns, r0 + 32);
-  for (int c = threadIdx.x; c < ws; c += kThreads) {
-    int e = 0;
-    for (int r = r0; r < r1; ++r) e = max(e, biased_exponent(Y[s.y_off + (int64_t)r * ws + c]));
-    if (e) atomicMax(&colexp[sd.col_off + s.jlo + c], e);
   }
 }
 
@@ -314,224 +305,225 @@ __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(
   }
 }
 
-// Sparse TRSM of one 32-column chunk with split-precision updates: the 32x32
-// diagonal triangles are solved in FP64 by one warp exactly as in the FP64
-// path; the update of the panel rows below (L[p, block] X, paper Sec. 3.2's
-// pruned GEMM) runs on the tensor cores from digit planes of X (column
-// bounds, shared memory) and of L's rows (pre-cut by lpack_kernel), combined
-// exactly in integers and subtracted from Y in FP64.
-template <int S>
-// 6 resident CTAs for up to 4 digits (the TRSM is latency-bound: more warps
-// hide the L digit and Y loads), 5 for 5 digits (at 6 its registers spill), 4 for
-// 6 and 7 digits (their fragments would spill)
-__global__ void __launch_bounds__(kThreads, (S <= 4 ? 6 : S == 5 ? 5 : 4)) trsm_split_kernel(const PlanPtrs P, const double *__restrict__ Lv,
-                                                              const double *__restrict__ invd,
-                                                              const __nv_bfloat16 *__restrict__ Ld,
-                                                              const int16_t *__restrict__ lexp, int64_t ld_rows,
-                                                              double *__restrict__ Y) {
-  __shared__ double Xs[32][33];
-  __shared__ int64_t cps[32];
-  __shared__ __align__(16) __nv_bfloat16 PX[S][32][kPad];   // digit planes of X, [t][column][row]
-  __shared__ int emaxX[32];
-  const TrsmTask t = P.trsm_tasks[blockIdx.x];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g = lane >> 2, tg = lane & 3;
-  const int c_hi = t.c_lo + t.w;
-  // the warp that solves the FP64 triangles: spread over the SM's sub-partitions
-  // across co-resident CTAs (a hash of the task index; see tri_warp in sc_kernels.cu)
-  const int tri = (int)(((unsigned)blockIdx.x * 2654435761u) >> 30);
+// ---- sparse TRSM with split-precision updates ------------------------------
+//
+// A CTA of four warps has 4 C columns of a 32-column chunk, C to a warp.  A warp
+// solves the triangles of its own columns in FP64 (sc_trsm.cuh), without waiting
+// for the others; the update of the rows below a block of more than kDirect columns
+// is the CTA's: its columns' digit planes in shared memory, the rows' m-tiles dealt to the
+// warps, each L fragment used for all of the CTA's columns.  Narrow CTAs (C = 2) have
+// the shorter triangles and fill the GPU on small batches; C is chosen as the FP64 TRSM's
+// columns per warp are (sc_plan.cpp).  Bound by the FP64 pipe (triangles, and two
+// operations per entry and block after the digit products) and by latency.  Against one CTA
+// per 32-column chunk whose warps shared each triangle 8 columns at a time, 7 digits, TRSM with its packing:
+// one square 312 -> 64 us, 36 squares 1.11 -> 0.33 ms, 8 elasticity cubes 4.04 -> 2.31 ms,
+// 64 heat cubes 6.05 -> 6.35 ms (their SYRK stage gains 0.14 ms: the columns' bounds come from here).
 
-  for (int li = 0; li < t.list_len; ++li) {
-    const SnDev s = P.sns[P.trsm_list[t.list_off + li]];
-    const int a = max(s.jlo, t.c_lo), b = min(s.jhi, c_hi), w = b - a, ws = s.jhi - s.jlo;
-    double *Ys = Y + s.y_off + (a - s.jlo);
-    const int total = s.ns * w;
-    for (int idx = tid; idx < total; idx += kThreads) {
-      const int r = idx / w, c = idx - r * w;
-      Ys[(int64_t)r * ws + c] = 0.0;
+struct TrsmSplit {
+  const __nv_bfloat16 *Ld;     // digit planes of L
+  const int16_t *lexp;         // its rows' exponent bounds
+  int64_t ld_rows;
+  int *colexp;                 // exponent bounds of Y's columns (out)
+};
+
+template <int C, int S>
+struct TeamShared {
+  TrsmShared<C> w[kThreads / 32];
+  double T[32 * 31 / 2];                            // a wide block's triangle over its diagonal, L(row, p) / L(p, p)
+  __align__(16) __nv_bfloat16 PX[S][4 * C][kPad];   // digit planes of the block's X: [digit][live column][row]
+  int emax[4 * C];                                  // and their columns' exponent bounds
+};
+
+template <int C, int S>
+__device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, int part, const double *__restrict__ Lv,
+                                          const double *__restrict__ invd, const TrsmSplit &sp,
+                                          double *__restrict__ Y, TeamShared<C, S> &sm, int warp, int lane) {
+  constexpr int kRows = 32 / C;                                    // rows of a block's X that a warp's lanes cover
+  const int g = lane >> 2, tg = lane & 3;
+  const int c_lo = t.c_lo + part * 4 * C, c_hi = min(c_lo + 4 * C, t.c_lo + t.w);
+  if (c_lo >= c_hi) return;                                        // uniform
+  const int w_lo = min(c_lo + warp * C, c_hi), w_hi = min(w_lo + C, c_hi);   // this warp's columns
+  TrsmShared<C> &own = sm.w[warp];
+  int *colexp = sp.colexp + P.subs[t.sub].col_off;
+  int n = 0;
+  for (int l0 = 0; l0 < t.list_len; l0 += 32) {
+    n = trsm_batch(P, t, l0, c_lo, c_hi, own.sn, lane);
+    for (int i = 0; i < n; ++i) {
+      const TrsmSn &s = own.sn[i];
+      const int j = w_lo + lane % C, ws = s.jhi - s.jlo;
+      if (j >= s.jlo && j < min(s.jhi, w_hi))
+        for (int r = lane / C; r < s.ns; r += kRows) Y[s.y_off + (int64_t)r * ws + j - s.jlo] = 0.0;
     }
   }
-  __syncthreads();
-  for (int e = t.seed_lo + tid; e < t.seed_hi; e += kThreads) {
-    const Seed sd = P.seeds[e];
-    Y[sd.y_off] = sd.value;
+  __syncwarp();
+  {
+    const int32_t *seed = P.seed_ptr + P.subs[t.sub].col_off;
+    const int e1 = seed[w_hi];
+    for (int e = seed[w_lo] + lane; e < e1; e += 32) Y[P.seeds[e].y_off] = P.seeds[e].value;
   }
-  __syncthreads();
+  __syncwarp();
 
-  for (int li = 0; li < t.list_len; ++li) {
-    const SnDev s = P.sns[P.trsm_list[t.list_off + li]];
-    const int a = max(s.jlo, t.c_lo), b = min(s.jhi, c_hi), ws = s.jhi - s.jlo;
-    double *Ys = Y + s.y_off + (a - s.jlo);
-    const int64_t *cp = P.lcp + s.lcp_off;
-    const double *id = invd + s.lcp_off;
-    const int64_t *rm = P.rmap + s.rmap_off;
-    const int colsh = a - s.jlo;
-    const int nrow = s.ns + s.rs;
-    for (int kb = 0, blk = 0; kb < s.ns; kb += 32, ++blk) {
-      const int kw = min(32, s.ns - kb);
-      const int wk = min(b, P.cuts[s.cut_off + (kb >> 5)]) - a;
-      if (wk <= 0) continue;
-      const int nb = nrow - (kb + kw);
-      const int64_t base = s.ld_off + (int64_t)blk * nrow - 16LL * blk * (blk + 1);
-      // the L digit fragments of a warp's first m-tile depend on L only: the
-      // warps that do not solve the triangle fetch them while it is solved
-      uint32_t afr[S][2][4];
-      auto load_afr = [&](int mt) {
-        const int ra = mt * 16 + g, rb = ra + 8;
-        const bool va = ra < nb, vb = rb < nb;
-#pragma unroll
-        for (int d = 0; d < S; ++d) {
-          const uint32_t *pa = reinterpret_cast<const uint32_t *>(Ld + (int64_t)d * ld_rows * 32 + (base + ra) * 32);
-          const uint32_t *pb = reinterpret_cast<const uint32_t *>(Ld + (int64_t)d * ld_rows * 32 + (base + rb) * 32);
-#pragma unroll
-          for (int ks = 0; ks < 2; ++ks) {
-            afr[d][ks][0] = va ? pa[8 * ks + tg] : 0u;
-            afr[d][ks][1] = vb ? pb[8 * ks + tg] : 0u;
-            afr[d][ks][2] = va ? pa[8 * ks + tg + 4] : 0u;
-            afr[d][ks][3] = vb ? pb[8 * ks + tg + 4] : 0u;
-          }
-        }
-      };
-      const bool pre = warp != tri && warp * 16 < nb;
-      if (pre) load_afr(warp);
-      // The FP64 triangle, 8 columns at a time: warp `tri` solves the 8x8
-      // diagonal piece, then all four warps update the block's rows below it
-      // (one warp alone would hold its sub-partition's FP64 unit for the whole
-      // chain of ~kw^2 / 2 instructions while the others wait).  Every entry
-      // gets its updates in the same column order as a column-by-column solve.
-      if (tid < kw) cps[tid] = cp[kb + tid] - (kb + tid);
-      for (int e = tid; e < kw * 32; e += kThreads) {
-        const int q = e >> 5, c = e & 31;
-        Xs[q][c] = c < wk ? Ys[(int64_t)(kb + q) * ws + c] : 0.0;
-      }
-      __syncthreads();
-      for (int p0 = 0; p0 < kw; p0 += 8) {
-        const int pe = min(p0 + 8, kw);
-        if (warp == tri && lane < wk) {
-          if (pe - p0 == 8) {                 // a full piece: its column of X in registers
-            double x[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = Xs[p0 + i][lane];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              x[i] *= id[kb + p0 + i];
-              const double *Lc = Lv + cps[p0 + i] + kb + p0;
-#pragma unroll
-              for (int r = i + 1; r < 8; ++r) x[r] = fma(-Lc[r], x[i], x[r]);
+  for (int l0 = 0; l0 < t.list_len; l0 += 32) {
+    if (t.list_len > 32) n = trsm_batch(P, t, l0, c_lo, c_hi, own.sn, lane);
+    for (int i = 0; i < n; ++i) {
+      const TrsmSn s = own.sn[i];
+      const int ws = s.jhi - s.jlo, nr = s.ns + s.rs;
+      const int a4 = max(s.jlo, c_lo), b4 = min(s.jhi, c_hi);      // the CTA's live columns
+      const int a = max(s.jlo, w_lo), b = min(s.jhi, w_hi);        // the warp's
+      const int64_t *rm = P.rmap + s.rmap_off;
+      const double *Lc = Lv + s.lval;
+      for (int kb = 0, blk = 0; kb < s.ns; kb += 32, ++blk) {
+        const int kw = min(32, s.ns - kb), below = kb + kw, nb = nr - below;
+        const int cut = P.cuts[s.cut_off + blk];
+        const int wk4 = min(b4, cut) - a4, wk = min(b, cut) - a;
+        if (wk4 > 0) {                                             // uniform
+          const bool team = kw > kDirect && nb > 0;
+          double *Ys = Y + s.y_off + (a - s.jlo);
+          int em = 0;
+          const double idv = lane < kw ? invd[s.lcp_off + kb + lane] : 0.0;
+          if (kw > kDirect) {                                      // the CTA's warps share the triangle
+#pragma unroll 4
+            for (int p = warp; p < kw; p += kThreads / 32) {
+              const double inv = __shfl_sync(0xffffffffu, idv, p);
+              // panel row kb + lane of column kb + p
+              if (lane > p && lane < kw) sm.T[tri_at(lane, p)] = Lc[kb + lane + p * (nr - kb - 1) - p * (p - 1) / 2] * inv;
             }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) Xs[p0 + i][lane] = x[i];
-          } else {
-            for (int q = p0; q < pe; ++q) {
-              const double xq = Xs[q][lane] * id[kb + q];
-              Xs[q][lane] = xq;
-              const double *Lc = Lv + cps[q];
-              for (int r = q + 1; r < pe; ++r) Xs[r][lane] = fma(-Lc[kb + r], xq, Xs[r][lane]);
+            __syncthreads();
+          }
+          if (wk > 0) {
+            if (kw > kDirect) {
+              trsm_triangle<C, true>(own, sm.T, Ys + (int64_t)kb * ws, ws, kw, wk, idv, lane);
+            } else {
+              trsm_stage_triangle(own, Lc, nr, kb, kw, lane);
+              asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+              __syncwarp();
+              trsm_triangle<C, false>(own, own.T, Ys + (int64_t)kb * ws, ws, kw, wk, idv, lane);
             }
+            __syncwarp();
+            // the columns' exponent bounds, for the digits of X and for Y's planes
+            if (lane % C < wk)
+              for (int r = lane / C; r < kw; r += kRows) em = max(em, biased_exponent(own.X[r][lane % C]));
+#pragma unroll
+            for (int d = C; d < 32; d <<= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, d));
+            if (lane < wk && em) atomicMax(colexp + a + lane, em);
           }
-        }
-        __syncthreads();
-        if (pe < kw) {                        // then pe == p0 + 8
-          if (lane < wk) {
-            double x[8];
+          if (team) {
+            if (wk > 0) {
+              const int cl = lane % C, cc = a - a4 + cl;
+              if (lane < wk) sm.emax[cc] = em;
+              if (cl < wk)
+                for (int r = lane / C; r < 32; r += kRows) {
+                  const double v = r < kw ? own.X[r][cl] : 0.0;
+                  const uint64_t m = fixed_point(v, em);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = Xs[p0 + i][lane];
-            for (int r = pe + ((warp - tri) & 3); r < kw; r += kThreads / 32) {
-              double xr = Xs[r][lane];
-#pragma unroll
-              for (int i = 0; i < 8; ++i) xr = fma(-Lv[cps[p0 + i] + kb + r], x[i], xr);
-              Xs[r][lane] = xr;
+                  for (int d = 0; d < S; ++d) sm.PX[d][cc][r] = digit_bf16(m, d, v < 0.0);
+                }
             }
-          }
-          __syncthreads();
-        }
-      }
-      if (warp == tri) {
-        int em = 0;
-        if (lane < wk) {
-          for (int q = 0; q < kw; ++q) {
-            Ys[(int64_t)(kb + q) * ws + lane] = Xs[q][lane];
-            em = max(em, biased_exponent(Xs[q][lane]));
-          }
-        }
-        emaxX[lane] = em;
-      }
-      __syncthreads();
-      if (nb <= 0) continue;                  // nothing below this block (uniform)
-      for (int e = tid; e < 32 * 32; e += kThreads) {
-        const int q = e >> 5, c = e & 31;
-        const double v = (q < kw && c < wk) ? Xs[q][c] : 0.0;
-        const uint64_t X = fixed_point(v, emaxX[c]);
-        const bool neg = v < 0.0;
+            __syncthreads();
+            const int64_t base = s.ld_off + (int64_t)blk * nr - 16LL * blk * (blk + 1);
+            const int colsh = a4 - s.jlo;
+            for (int r0 = 16 * warp; r0 < nb; r0 += 16 * (kThreads / 32)) {
+              const int ra = r0 + g, rb = r0 + g + 8;
+              const bool va = ra < nb, vb = rb < nb;
+              uint4 fa[S], fb[S];
 #pragma unroll
-        for (int d = 0; d < S; ++d) PX[d][c][q] = digit_bf16(X, d, neg);
-      }
-      __syncthreads();
-      for (int mt = warp; mt * 16 < nb; mt += kThreads / 32) {
-        const int r0 = mt * 16;               // first block row of this m-tile
-        const int ra = r0 + g, rb = r0 + g + 8;
-        const bool va = ra < nb, vb = rb < nb;
-        const int ea = va ? lexp[base + ra] : 0, eb = vb ? lexp[base + rb] : 0;
-        // this lane's two target rows (a pruned row through its map), looked up once per m-tile
-        double *tga = nullptr, *tgb = nullptr;
-        if (va) {
-          const int p = kb + kw + ra;
-          tga = (p < s.ns) ? (Ys + (int64_t)p * ws) : (Y + rm[p - s.ns] + colsh);
-        }
-        if (vb) {
-          const int p = kb + kw + rb;
-          tgb = (p < s.ns) ? (Ys + (int64_t)p * ws) : (Y + rm[p - s.ns] + colsh);
-        }
-        if (!(pre && mt == warp)) load_afr(mt);
+              for (int d = 0; d < S; ++d) {
+                const uint4 *pl = reinterpret_cast<const uint4 *>(sp.Ld + (int64_t)d * sp.ld_rows * 32) + (base + ra) * 4 + tg;
+                fa[d] = va ? pl[0] : make_uint4(0u, 0u, 0u, 0u);
+                fb[d] = vb ? pl[32] : make_uint4(0u, 0u, 0u, 0u);
+              }
+              const int ea = va ? sp.lexp[base + ra] : 0, eb = vb ? sp.lexp[base + rb] : 0;
+              double *ta = nullptr, *tb = nullptr;                 // this lane's two target rows
+              if (va) ta = Y + colsh + (below + ra < s.ns ? s.y_off + (int64_t)(below + ra) * ws : rm[below + ra - s.ns]);
+              if (vb) tb = Y + colsh + (below + rb < s.ns ? s.y_off + (int64_t)(below + rb) * ws : rm[below + rb - s.ns]);
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-          if (8 * nt >= wk) break;                   // uniform across the warp
-          // the targets' current values, loaded before the products so that
-          // their latency overlaps the MMAs
-          double yv[4];
+              for (int nt = 0; nt < C / 2; ++nt) {
+                if (8 * nt >= wk4) break;                          // uniform
+                // the targets' current values, loaded before the products so that
+                // their latency overlaps the MMAs
+                double yv[4];
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const bool vr = (r & 2) ? vb : va;
-            const int col = 8 * nt + 2 * tg + (r & 1);
-            yv[r] = (vr && col < wk) ? ((r & 2) ? tgb : tga)[col] : 0.0;
-          }
-          Groups<S> gr[4];
+                for (int r = 0; r < 4; ++r) {
+                  const int col = 8 * nt + 2 * tg + (r & 1);
+                  const double *p = (r & 2) ? tb : ta;
+                  yv[r] = (p && col < wk4) ? p[col] : 0.0;
+                }
+                Groups<S> gr[4];
 #pragma unroll
-          for (int d = 0; d < S; ++d) {
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int d = 0; d < S; ++d) {
+                  float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int ta = 0; ta <= d; ++ta) {
-              const int tb = d - ta;
+                  for (int q = 0; q <= d; ++q) {
+                    const __nv_bfloat16 *px = &sm.PX[d - q][8 * nt + g][2 * tg];
+                    const uint32_t a0[4] = {fa[q].x, fb[q].x, fa[q].y, fb[q].y};
+                    const uint32_t a1[4] = {fa[q].z, fb[q].z, fa[q].w, fb[q].w};
+                    mma_bf16(c, a0, ld_pair(px), ld_pair(px + 8));
+                    mma_bf16(c, a1, ld_pair(px + 16), ld_pair(px + 24));
+                  }
 #pragma unroll
-              for (int ks = 0; ks < 2; ++ks) {
-                const uint32_t b0 = ld_pair(&PX[tb][8 * nt + g][16 * ks + 2 * tg]);
-                const uint32_t b1 = ld_pair(&PX[tb][8 * nt + g][16 * ks + 2 * tg + 8]);
-                mma_bf16(c, afr[ta][ks], b0, b1);
+                  for (int r = 0; r < 4; ++r) gr[r].add(d, __float2int_rn(c[r]));
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                  const int col = 8 * nt + 2 * tg + (r & 1);
+                  double *p = (r & 2) ? tb : ta;
+                  if (p && col < wk4) {
+                    // one conversion and one FMA on the FP64 pipe: both power-of-two
+                    // scalings folded into a single exponent
+                    const int e = ((r & 2 ? eb : ea) - 1022) + (sm.emax[col] - 1022) + Groups<S>::kBlockShift;
+                    const double v = (double)gr[r].block_int();
+                    p[col] = (e >= -1022 && e <= 1023) ? fma(-v, pow2i(e), yv[r]) : yv[r] - ldexp(v, e);
+                  }
+                }
               }
             }
+            __syncthreads();
+          } else if (kw > kDirect) {
+            __syncthreads();                                       // T is read by all
+          } else if (wk > 0) {
+            // FP64 update of the warp's own columns: (row, column) pairs, four to a lane
+            const int dp = 32 / wk, cl = lane % wk;
+            for (int p0 = below + (lane < dp * wk ? lane / wk : nr); __any_sync(0xffffffffu, p0 < nr); p0 += 4 * dp) {
+              int row[4];
+              const int col[4] = {cl, cl, cl, cl};
+              double *tg4[4];
+              double acc[4];
+              int last = 0;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) gr[r].add(d, __float2int_rn(c[r]));
-          }
+              for (int j = 0; j < 4; ++j) {
+                const int p = p0 + j * dp;
+                const bool ok = p < nr;
+                if (__any_sync(0xffffffffu, ok)) last = j + 1;
+                row[j] = ok ? p : nr - 1;
+                tg4[j] = !ok ? nullptr : (p < s.ns ? Ys + (int64_t)p * ws : Y + rm[p - s.ns] + (a - s.jlo)) + cl;
+                acc[j] = ok ? *tg4[j] : 0.0;
+              }
+              if (last <= 1) trsm_update<1, false>(own, Lc, nr, kb, kw, row, col, acc);
+              else if (last <= 2) trsm_update<2, false>(own, Lc, nr, kb, kw, row, col, acc);
+              else trsm_update<4, false>(own, Lc, nr, kb, kw, row, col, acc);
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const bool vr = (r & 2) ? vb : va;
-            const int col = 8 * nt + 2 * tg + (r & 1);
-            if (vr && col < wk) {
-              const int e = (((r & 2) ? eb : ea) - 1022) + (emaxX[col] - 1022);
-              // one conversion and one FMA on the FP64 pipe: both power-of-two
-              // scalings folded into a single exponent
-              const double v = (double)gr[r].block_int();
-              const int eb = e + Groups<S>::kBlockShift;
-              double *tgt = (r & 2) ? tgb : tga;
-              if (eb >= -1022 && eb <= 1023) tgt[col] = fma(-v, pow2i(eb), yv[r]);
-              else tgt[col] = yv[r] - ldexp(v, eb);
+              for (int j = 0; j < 4; ++j)
+                if (tg4[j]) *tg4[j] = acc[j];
             }
+            __syncwarp();
           }
         }
+        Lc += 32LL * (nr - kb) - 16 * 33;                          // panel row t of column kb + 32
       }
-      __syncthreads();
     }
   }
+}
+
+// Resident CTAs: with C = 2 three (168 registers, no spills: 2.9 -> 2.3 ms on eight elasticity cubes at 7 digits),
+// with C = 4 four (6.6 -> 6.3 ms on 64 heat cubes).
+template <int C, int S>
+__global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(const PlanPtrs P, const double *__restrict__ Lv,
+                                                              const double *__restrict__ invd, const TrsmSplit sp,
+                                                              double *__restrict__ Y) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  constexpr int kParts = kChunk / (4 * C);
+  trsm_team<C, S>(P, P.trsm_tasks[blockIdx.x / kParts], blockIdx.x % kParts, Lv, invd, sp, Y,
+                  *reinterpret_cast<TeamShared<C, S> *>(team_smem), threadIdx.x >> 5, threadIdx.x & 31);
 }
 
 }  // namespace
@@ -560,16 +552,27 @@ int launch_lpack_split(const sc_ctx &c, int S_, int64_t base, int64_t count, con
   return (int)cudaGetLastError();
 }
 
-int launch_trsm_split(const sc_ctx &c, int S_, int64_t base, int64_t count, const double *Lv, const double *invd,
-                      void *ws, double *Y, void *stream) {
+template <int C, int S>
+static void launch_team(const PlanPtrs &p, int n, const double *Lv, const double *invd, const TrsmSplit &sp, double *Y,
+                        cudaStream_t st) {
+  const int smem = (int)sizeof(TeamShared<C, S>);
+  cudaFuncSetAttribute(trsm_split_kernel<C, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  trsm_split_kernel<C, S><<<(unsigned)(n * (kChunk / (4 * C))), kThreads, smem, st>>>(p, Lv, invd, sp, Y);
+}
+
+int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t count, const double *Lv,
+                      const double *invd, void *ws, double *Y, void *stream) {
   if (count <= 0) return (int)cudaGetLastError();
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t *w = static_cast<uint8_t *>(ws);
-  const __nv_bfloat16 *Ld = reinterpret_cast<const __nv_bfloat16 *>(w + c.ws.ld_off);
-  const int16_t *lexp = reinterpret_cast<const int16_t *>(w + c.ws.lexp_off);
+  const TrsmSplit sp{reinterpret_cast<const __nv_bfloat16 *>(w + c.ws.ld_off),
+                     reinterpret_cast<const int16_t *>(w + c.ws.lexp_off), c.ws.ld_rows,
+                     reinterpret_cast<int *>(w + c.ws.colexp_off)};
   PlanPtrs p = c.ptrs();
   p.trsm_tasks += base;
-#define TS(S) trsm_split_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, Ld, lexp, c.ws.ld_rows, Y)
+#define TS(S)                                                                       \
+  if (cols >= 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);       \
+  else launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st)
   SC_SPLIT_SWITCH(S_, TS)
 #undef TS
   return (int)cudaGetLastError();
@@ -588,11 +591,10 @@ int launch_yslice_group(const sc_ctx &c, int S_, int64_t base, int64_t count, co
   if (count <= 0) return (int)cudaGetLastError();
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t *w = static_cast<uint8_t *>(ws);
-  int *colexp = reinterpret_cast<int *>(w + c.ws.colexp_off);
+  const int *colexp = reinterpret_cast<const int *>(w + c.ws.colexp_off);
   __nv_bfloat16 *Yd = reinterpret_cast<__nv_bfloat16 *>(w + c.ws.yd_off);
   PlanPtrs p = c.ptrs();
   p.sblk += 2 * base;
-  ycolexp_kernel<<<(unsigned)count, kThreads, 0, st>>>(p, Y, colexp);
 #define YS(S) yslice_kernel<S, false><<<(unsigned)count, kThreads, 0, st>>>(p, Y, colexp, Yd, c.ws.yd_plane)
 #define YB(S) yslice_kernel<S, true><<<(unsigned)count, kThreads, 0, st>>>(p, Y, colexp, Yd, c.ws.yd_plane)
   if (balanced) {
