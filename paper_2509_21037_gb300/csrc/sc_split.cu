@@ -172,20 +172,40 @@ __global__ void __launch_bounds__(kThreads) yslice_kernel(const PlanPtrs P, cons
   }
 }
 
+constexpr int kSyrkBatch = 64;   // supernodes whose rows are numbered through at a time
+
+// Y's digit rows that are live on a task's chunks, in units of 8 (a 16-byte copy per column and plane)
+struct SyrkUnits {
+  int64_t off[kSyrkBatch];             // digit offset of (first live row, sorted column 0)
+  int start[kSyrkBatch + 1];           // first unit of every supernode of the batch
+  int npad[kSyrkBatch], jlo[kSyrkBatch], jhi[kSyrkBatch];
+  int wsum;
+};
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
 // One 32x32 block of F = Y^T Y (sorted chunks q1 >= q2) from Y's digit
 // planes.  Warp w computes rows 16*(w>>1).. and columns 16*(w&1).. of the
-// block as two m16n8 tiles.
+// block as two m16n8 tiles.  The live rows of all listed supernodes are numbered
+// through in units of 8 and taken four units at a time (K = 32), whatever
+// supernodes they belong to; the next four are copied asynchronously meanwhile.
+// Bound by mma.sync issue (2.3 ms for 64 heat cubes at 7 digits).  Against one stage per supernode block and
+// word loads of the fragments, SYRK with its slicing, 7 digits: 64 heat cubes 5.84 -> 5.15 ms, 8
+// elasticity cubes 1.15 -> 1.08 ms, 36 squares 328 -> 135 us, one square 140 -> 41 us.
 template <int S>
 // 4 resident CTAs for up to 5 digits, 3 for 6 and 7 (register-bound fragments)
 __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(const PlanPtrs P, const __nv_bfloat16 *__restrict__ Yd,
                                                               int64_t yd_plane, const int *__restrict__ colexp,
                                                               double *__restrict__ F) {
-  // two stages of the digit tiles: [stage][operand][t][column][k]; the next
-  // active 32-row block is fetched with asynchronous copies while this one
-  // is multiplied
+  // two stages of the digit tiles: [stage][operand][t][column][k]
   extern __shared__ __align__(16) unsigned char syrk_smem[];
   typedef __nv_bfloat16 Tile[S][32][kPad];
   Tile *stages = reinterpret_cast<Tile *>(syrk_smem);          // stages[2 * buf + op]
+  __shared__ SyrkUnits un;
   const SyrkTask t = P.syrk_tasks[blockIdx.x];
   const SubDev sd = P.subs[t.sub];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -193,56 +213,85 @@ __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(
   const int j1lo = t.q1 * kChunk, j2lo = t.q2 * kChunk;
   const int mrow = 16 * (warp >> 1), ncol = 16 * (warp & 1);
   // per output: the Horner words of the digit-group sums, accumulated over
-  // blocks (linear, exact: < 128 blocks * 2^24 * 256^(h-1) < 2^63)
+  // stages (linear, exact: < 128 stages * 2^24 * 256^(h-1) < 2^63)
   Groups<S> acc[8];
   double dacc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) dacc[i] = 0.0;
   int blocks = 0;
-  // the active (supernode, 32-row block) pairs in order: rows of a supernode
-  // at or after its pivot cut for this chunk are zero and skipped
-  auto advance = [&](int &li, int &k0) -> bool {
-    for (;;) {
-      k0 += 32;
-      while (li < t.list_len && k0 >= P.sns[P.syrk_list[t.list_off + li]].ns) {
-        ++li;
-        k0 = 0;
-      }
-      if (li >= t.list_len) return false;
-      const SnDev &sn = P.sns[P.syrk_list[t.list_off + li]];
-      if (j1lo < P.cuts[sn.cut_off + (k0 >> 5)]) return true;
+  for (int l0 = 0; l0 < t.list_len; l0 += kSyrkBatch) {
+    int n = 0;
+    if (tid < kSyrkBatch && l0 + tid < t.list_len) {
+      const SnDev s = P.sns[P.syrk_list[t.list_off + l0 + tid]];
+      const int nb = (s.ns + 31) >> 5;
+      int b = 0;
+      while (b < nb && P.cuts[s.cut_off + b] <= j1lo) ++b;     // rows before the first live block are zero on q1
+      n = max(0, s.ns - 32 * b + 7) >> 3;
+      const int npad = 32 * nb;
+      un.npad[tid] = npad;
+      un.off[tid] = s.yd_off - (int64_t)s.jlo * npad + 32 * b;
+      un.jlo[tid] = s.jlo;
+      un.jhi[tid] = s.jhi;
     }
-  };
-  // 2 operands x S planes x 32 columns x 4 vectors of 8 digits, 16 bytes each
-  auto fetch = [&](int li, int k0, int buf) {
-    const SnDev sn = P.sns[P.syrk_list[t.list_off + li]];
-    const int npad = (sn.ns + 31) / 32 * 32;
-    for (int v = tid; v < 2 * S * 32 * 4; v += kThreads) {
-      const int part = v & 3, col = (v >> 2) & 31, d = (v >> 7) % S, op = (v >> 7) / S;
-      const int j = (op == 0 ? j1lo : j2lo) + col - sn.jlo;
-      const bool in = j >= 0 && j < sn.jhi - sn.jlo;
-      const __nv_bfloat16 *src =
-          in ? Yd + (int64_t)d * yd_plane + sn.yd_off + (int64_t)j * npad + k0 + 8 * part : Yd;
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&stages[2 * buf + op][d][col][8 * part]);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 16 : 0)
-                   : "memory");
+    int inc = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= d) inc += v;
     }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  };
-  int li = 0, k0 = -32, buf = 0;
-  bool have = advance(li, k0);
-  if (have) fetch(li, k0, 0);
-  while (have) {
-    int nli = li, nk0 = k0;
-    const bool nhave = advance(nli, nk0);
-    if (nhave) {
-      fetch(nli, nk0, buf ^ 1);
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");   // this block's copies are done
-    } else {
-      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    }
+    if (tid == 31) un.wsum = inc;
     __syncthreads();
-    const Tile &PA = stages[2 * buf], &PB = stages[2 * buf + 1];
+    if (tid < kSyrkBatch) un.start[tid + 1] = inc + (warp == 1 ? un.wsum : 0);
+    if (tid == 0) un.start[0] = 0;
+    __syncthreads();
+    const int total = un.start[kSyrkBatch];
+    // this thread copies unit `part` of column `col` of every stage, all planes of both operands
+    const int part = tid & 3, col = tid >> 2;
+    auto fetch = [&](int st) {
+      const int u = 4 * st + part;
+      const __nv_bfloat16 *src[2] = {Yd, Yd};
+      int bytes[2] = {0, 0};
+      if (u < total) {
+        int e = 0;
+#pragma unroll
+        for (int h = kSyrkBatch / 2; h >= 1; h >>= 1)
+          if (un.start[e + h] <= u) e += h;
+        const int64_t off = un.off[e] + 8 * (u - un.start[e]);
+#pragma unroll
+        for (int op = 0; op < 2; ++op) {
+          const int j = (op == 0 ? j1lo : j2lo) + col;
+          if (j >= un.jlo[e] && j < un.jhi[e]) {
+            src[op] = Yd + off + (int64_t)j * un.npad[e];
+            bytes[op] = 16;
+          }
+        }
+      }
+#pragma unroll
+      for (int op = 0; op < 2; ++op) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&stages[2 * (st & 1) + op][0][col][8 * part]);
+        const int64_t step = bytes[op] ? yd_plane : 0;
+#pragma unroll
+        for (int d = 0; d < S; ++d)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + (uint32_t)(d * 32 * kPad * 2)),
+                       "l"(src[op] + d * step), "r"(bytes[op])
+                       : "memory");
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    const int nst = (total + 3) >> 2;
+    if (nst > 0) fetch(0);
+    for (int st = 0; st < nst; ++st) {
+      if (st + 1 < nst) {
+        fetch(st + 1);
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");   // this stage's copies are done
+      } else {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+      }
+      __syncthreads();
+      const Tile &PA = stages[2 * (st & 1)], &PB = stages[2 * (st & 1) + 1];
+      // rows of the fragments that this lane's ldmatrix address names
+      const int ar = mrow + (lane & 15), ak = 8 * (lane >> 4);
+      const int br = ncol + (lane & 7) + 8 * (lane >> 4), bk = 8 * ((lane >> 3) & 1);
 #pragma unroll
       for (int d = 0; d < S; ++d) {
         float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
@@ -251,17 +300,11 @@ __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(
           const int tb = d - ta;
 #pragma unroll
           for (int ks = 0; ks < 32; ks += 16) {
-            uint32_t a[4];
-            a[0] = ld_pair(&PA[ta][mrow + g][ks + 2 * tg]);
-            a[1] = ld_pair(&PA[ta][mrow + g + 8][ks + 2 * tg]);
-            a[2] = ld_pair(&PA[ta][mrow + g][ks + 2 * tg + 8]);
-            a[3] = ld_pair(&PA[ta][mrow + g + 8][ks + 2 * tg + 8]);
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-              const uint32_t b0 = ld_pair(&PB[tb][ncol + 8 * nt + g][ks + 2 * tg]);
-              const uint32_t b1 = ld_pair(&PB[tb][ncol + 8 * nt + g][ks + 2 * tg + 8]);
-              mma_bf16(c[nt], a, b0, b1);
-            }
+            uint32_t a[4], b[4];
+            ldmatrix_x4(a, &PA[ta][ar][ks + ak]);
+            ldmatrix_x4(b, &PB[tb][br][ks + bk]);
+            mma_bf16(c[0], a, b[0], b[1]);
+            mma_bf16(c[1], a, b[2], b[3]);
           }
         }
 #pragma unroll
@@ -269,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(
 #pragma unroll
           for (int r = 0; r < 4; ++r) acc[nt * 4 + r].accumulate(d, __float2int_rn(c[nt][r]));
       }
-      __syncthreads();                // the next iteration's fetch overwrites this stage
+      __syncthreads();                // the next fetch overwrites this stage (or the next batch the units)
       if (++blocks == 128) {          // int64 headroom, see acc
         blocks = 0;
 #pragma unroll
@@ -278,10 +321,7 @@ __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(
           acc[i] = Groups<S>();
         }
       }
-    li = nli;
-    k0 = nk0;
-    have = nhave;
-    buf ^= 1;
+    }
   }
   const int32_t *perm = P.perm_cols + sd.col_off;
   const int *ce = colexp + sd.col_off;
