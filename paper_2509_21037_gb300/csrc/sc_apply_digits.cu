@@ -43,6 +43,7 @@
 #include <string>
 
 #include "sc_internal.h"
+#include "sc_tiles.cuh"
 
 using namespace sc;
 
@@ -85,15 +86,14 @@ __device__ __forceinline__ long long fixed55(double x, int emax) {
   return (b >> 63) ? -(long long)m : (long long)m;
 }
 
-// balanced base-256 digits of M (|M| <= 2^54), most significant first, in
-// offset binary: ob[k] = d_k + 128
+// Balanced base-256 digits of M (|M| <= 2^54), most significant first: M = sum_k d_k 256^(6-k) makes
+// M + sum_k 128 256^(6-k) the number whose base-256 digits are d_k + 128.
+constexpr unsigned long long kOffsetBytes = 0x80808080808080ull;
+
 __device__ __forceinline__ void digits7(long long M, int (&d)[kDigitsF]) {
+  const unsigned long long u = (unsigned long long)M + kOffsetBytes;
 #pragma unroll
-  for (int k = kDigitsF - 1; k >= 0; --k) {
-    const int v = (int)((M + 128) & 255) - 128;
-    d[k] = v;
-    M = (M - v) >> 8;
-  }
+  for (int k = 0; k < kDigitsF; ++k) d[k] = (int)((u >> (8 * (6 - k))) & 255) - 128;
 }
 
 // 2^e as a double, also outside the normal range
@@ -122,7 +122,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 }
 
 // ---------------------------------------------------------------------------
-// Digit form of F: one warp per tile; lane r holds row r.
+// Digit form of F: one warp per tile; lane r holds row r.  Bound by HBM and by the integer operations of the cut
+// to fixed point: 136 us for 53306 tiles (0.82 GB, 6.0 TB/s); with the digits taken out one by one 238 us.
 __global__ void __launch_bounds__(kPrepWarps * 32) digits_prepare_kernel(const double *__restrict__ F,
                                                                         unsigned char *__restrict__ Fd,
                                                                         int64_t n_tiles) {
@@ -142,29 +143,21 @@ __global__ void __launch_bounds__(kPrepWarps * 32) digits_prepare_kernel(const d
   const int R = lane >> 1, odd = lane & 1;
 #pragma unroll
   for (int C = 0; C < 16; ++C) {
-    int d0[kDigitsF], d1[kDigitsF];
-    digits7(fixed55(x[2 * C], emax), d0);
-    digits7(fixed55(x[2 * C + 1], emax), d1);
-    // this row's bytes of columns 2C, 2C+1 for each digit, two digits per 32-bit word
-    uint32_t h[4];
+    // the digits in offset binary are the low seven bytes of M + kOffsetBytes, digit k byte 6 - k
+    const unsigned long long m0 = (unsigned long long)fixed55(x[2 * C], emax) + kOffsetBytes;
+    const unsigned long long m1 = (unsigned long long)fixed55(x[2 * C + 1], emax) + kOffsetBytes;
+    const uint32_t w[4] = {(uint32_t)m0, (uint32_t)(m0 >> 32), (uint32_t)m1, (uint32_t)(m1 >> 32)};
+    uint32_t o[4];                    // the row of the other parity
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int k0 = 2 * p, k1 = 2 * p + 1;
-      const uint32_t lo = (uint32_t)(d0[k0] + 128) | ((uint32_t)(d1[k0] + 128) << 8);
-      const uint32_t hi = k1 < kDigitsF ? ((uint32_t)(d0[k1] + 128) | ((uint32_t)(d1[k1] + 128) << 8)) : 0u;
-      h[p] = lo | (hi << 16);
-    }
-    uint32_t o[4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) o[p] = __shfl_xor_sync(kFull, h[p], 1);
+    for (int p = 0; p < 4; ++p) o[p] = __shfl_xor_sync(kFull, w[p], 1);
     if ((C & 1) == odd) {
-      // even row's bytes (2R, 2C), (2R, 2C+1) and odd row's (2R+1, 2C), (2R+1, 2C+1)
 #pragma unroll
       for (int k = 0; k < kDigitsF; ++k) {
-        const int p = k >> 1, s = (k & 1) * 16;
-        const uint32_t ev = ((odd ? o[p] : h[p]) >> s) & 0xFFFFu;
-        const uint32_t ov = ((odd ? h[p] : o[p]) >> s) & 0xFFFFu;
-        wsm[warp][k * kPlaneWords + widx(R, C)] = prmt(ev, ov, 0x5140);   // x00 x10 x01 x11
+        const int h = (6 - k) >> 2, byte = (6 - k) & 3;
+        const uint32_t sel = (uint32_t)(byte | (4 + byte) << 4);            // byte of the even row, byte of the odd row
+        const uint32_t c0 = odd ? prmt(o[h], w[h], sel) : prmt(w[h], o[h], sel);
+        const uint32_t c1 = odd ? prmt(o[2 + h], w[2 + h], sel) : prmt(w[2 + h], o[2 + h], sel);
+        wsm[warp][k * kPlaneWords + widx(R, C)] = prmt(c0, c1, 0x5410);      // x00 x10 x01 x11
       }
     }
   }
@@ -188,6 +181,8 @@ __global__ void __launch_bounds__(kLamWarps * 32) digits_lambda_kernel(const Pla
                                                                       const double *__restrict__ lam,
                                                                       unsigned char *__restrict__ tab,
                                                                       double *__restrict__ q, int64_t n_dual) {
+  // the product may be launched now: it reads F's tiles ahead and waits for this grid before the rest
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_dual; i += (int64_t)gridDim.x * blockDim.x)
     q[i] = 0.0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -222,12 +217,6 @@ __global__ void __launch_bounds__(kLamWarps * 32) digits_lambda_kernel(const Pla
   if (lane == 0) reinterpret_cast<int *>(ent + kLamCjOff + 32)[0] = emax;
 }
 
-// the first tile of apply task k (storage order: subdomain, row block I, J = 0..I)
-__device__ __forceinline__ int64_t task_tile0(const PlanPtrs &P, int64_t k) {
-  const ApplyTask a = P.apply_tasks[k];
-  return P.subs[a.sub].F_off / 1024 + (int64_t)a.I * (a.I + 1) / 2;
-}
-
 // exact integer of an FP32 accumulator (subnormal-offset form) for class constant c
 __device__ __forceinline__ int acc_int(float d, float c) {
   return __float_as_int(__fmaf_rn(d, 16777216.0f, c)) - 0x4B400000;
@@ -258,24 +247,6 @@ __device__ __forceinline__ long long class_sum(const float (&d)[2][4], float c0,
   return k;
 }
 
-struct TileCursor {
-  int64_t task;
-  int sub, I, J, m;
-  __device__ __forceinline__ void load(const PlanPtrs &P) {
-    const ApplyTask a = P.apply_tasks[task];
-    sub = a.sub;
-    I = a.I;
-    m = P.subs[a.sub].m;
-  }
-  __device__ __forceinline__ void next(const PlanPtrs &P) {
-    if (++J > I) {
-      ++task;
-      J = 0;
-      load(P);
-    }
-  }
-};
-
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar));
 }
@@ -296,13 +267,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long lo
 
 // tile `tile` and the lambda block of task `lam_entry` into a stage: two bulk
 // copies completing on the stage's mbarrier (one thread)
-__device__ __forceinline__ void fetch_stage(uint32_t stage, uint32_t bar, const unsigned char *Fd,
-                                            const unsigned char *tab, int64_t tile, int64_t lam_entry) {
+__device__ __forceinline__ void fetch_tile(uint32_t stage, uint32_t bar, const unsigned char *Fd, int64_t tile) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kStageBytes) : "memory");
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                    stage),
                "l"(Fd + tile * kTileBytes), "r"(kTileBytes), "r"(bar)
                : "memory");
+}
+__device__ __forceinline__ void fetch_lambda(uint32_t stage, uint32_t bar, const unsigned char *tab, int64_t lam_entry) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                    stage + kTileBytes),
                "l"(tab + lam_entry * kLamBytes), "r"(kLamBytes), "r"(bar)
@@ -343,20 +315,18 @@ __global__ void __launch_bounds__(kPairs * 64, 1) apply_digits_kernel(const Plan
     abort_flag[pair] = 0;
   }
   asm volatile("bar.sync %0, 64;\n" ::"r"(1 + pair) : "memory");
-  int64_t lo = 0, hi = n_tasks - 1;               // the task holding tile t0
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) / 2;
-    if (task_tile0(P, mid) <= t0) lo = mid;
-    else hi = mid - 1;
-  }
-  TileCursor cur{lo, 0, 0, 0, 0};
-  cur.load(P);
-  cur.J = (int)(t0 - task_tile0(P, lo));
+  TileCursor cur = tile_at(P, n_tasks, t0);
   TileCursor pre = cur;                           // the next tile to fetch (issuing warp)
   const int64_t ntile = t1 - t0;
   if (half == 0) {
+    for (int s = 0; s < kStages - 1 && s < ntile; ++s)
+      if (issuer) fetch_tile(ring + s * kStageBytes, bar0 + 8 * s, Fd, t0 + s);
+  }
+  // F's first tiles are on their way; from here on what the lambda kernel wrote is read (and q added to)
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  if (half == 0) {
     for (int s = 0; s < kStages - 1 && s < ntile; ++s) {
-      if (issuer) fetch_stage(ring + s * kStageBytes, bar0 + 8 * s, Fd, tab, t0 + s, pre.task - pre.I + pre.J);
+      if (issuer) fetch_lambda(ring + s * kStageBytes, bar0 + 8 * s, tab, pre.task - pre.I + pre.J);
       if (s + 1 < ntile) pre.next(P);             // only within the range: the next task exists
     }
   }
@@ -397,8 +367,10 @@ __global__ void __launch_bounds__(kPairs * 64, 1) apply_digits_kernel(const Plan
     }
     const int sp = s == 0 ? kStages - 1 : s - 1;  // the stage of tile n - 1: refill with tile n + kStages - 1
     if (half == 0 && n + kStages - 1 < ntile) {
-      if (issuer) fetch_stage(ring + sp * kStageBytes, bar0 + 8 * sp, Fd, tab, t0 + n + kStages - 1,
-                              pre.task - pre.I + pre.J);
+      if (issuer) {
+        fetch_tile(ring + sp * kStageBytes, bar0 + 8 * sp, Fd, t0 + n + kStages - 1);
+        fetch_lambda(ring + sp * kStageBytes, bar0 + 8 * sp, tab, pre.task - pre.I + pre.J);
+      }
       if (n + kStages < ntile) pre.next(P);
     }
     const unsigned char *stage = dsm + (size_t)pair * kStages * kStageBytes + (size_t)s * kStageBytes;
@@ -543,10 +515,20 @@ extern "C" sc_status sc_apply_digits(sc_ctx *ctx, void *Fd_dev, const double *la
       if (e == cudaSuccess) {
         const int64_t grid = std::min<int64_t>(sms, (nt + kPairs - 1) / kPairs);
         const long long limit = ctx->poll_limit > 0 ? (long long)ctx->poll_limit : (1LL << 26);
-        apply_digits_kernel<<<(unsigned)grid, kPairs * 64, smem, st>>>(
-            ctx->ptrs(), ctx->n_apply, nt, Fd, tab, q_dev, reinterpret_cast<uint32_t *>(Fd + status_offset(ctx)),
-            limit);
-        e = cudaGetLastError();
+        // launched while the lambda kernel still runs (see griddepcontrol in both)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(kPairs * 64);
+        cfg.dynamicSmemBytes = (size_t)smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, apply_digits_kernel, ctx->ptrs(), (int64_t)ctx->n_apply, nt,
+                               (const unsigned char *)Fd, (const unsigned char *)tab, q_dev,
+                               reinterpret_cast<uint32_t *>(Fd + status_offset(ctx)), limit);
       }
     }
   }
