@@ -20,10 +20,12 @@
 // and tile, the size of an FP64 GEMV's rounding.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <string>
 
 #include "sc_internal.h"
+#include "sc_tiles.cuh"
 
 using namespace sc;
 
@@ -63,85 +65,180 @@ __device__ __forceinline__ void mac(long long &d0, long long &d1, long long &d2,
   d2 += (long long)m.y * l.y;
 }
 
-// fp64_quarters (0..4): of every four tiles a warp visits, this many are
-// multiplied in FP64 (FP64 pipe) and the rest in fixed point (integer pipes),
-// so that both pipes work at once; 0 is the pure fixed-point product.
-__global__ void __launch_bounds__(kThreads, 6) apply_fixed_kernel(const PlanPtrs P, const double *__restrict__ F,
-                                                               const double *__restrict__ lam,
-                                                               double *__restrict__ q, int fp64_quarters) {
-  __shared__ double Ts[kThreads / 32][32][33];     // the tile, then its limbs in place
-  __shared__ int2 LJ[kThreads / 32][32];           // limbs of the lambda block J
-  __shared__ int2 LI[kThreads / 32][32];           // limbs of the lambda block I
-  __shared__ double red[kThreads / 32][32];
-  const ApplyTask t = P.apply_tasks[blockIdx.x];
-  const SubDev sd = P.subs[t.sub];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int32_t *map = P.lambda + sd.col_off;
-  const int I = t.I;
-  const int rowI = I * kTile + lane;
-  const double pI = rowI < sd.m ? lam[map[rowI]] : 0.0;
-  const uint32_t exI = __reduce_max_sync(kFull, exp_field(pI));
-  LI[warp][lane] = fixed_limbs(pI, exI);
-  int2 *Tl = reinterpret_cast<int2 *>(&Ts[warp][0][0]);
-  double y = 0.0;
-  for (int J = warp; J <= I; J += kThreads / 32) {
-    const double *Tg = F + sd.F_off + ((int64_t)I * (I + 1) / 2 + J) * (kTile * kTile);
-    // stage the tile in shared memory (column c, row lane), eight loads in flight
-    // at a time, so that no lane keeps the whole tile in registers
-    uint32_t em = 0;
+constexpr int kStride = 34;                        // doubles between a tile's columns in shared memory (16-byte rows)
+constexpr int kApplyWarps = 4;                     // warps per CTA
+
+// In FP64 two stages per warp and 12 warps per SM: a warp's next tile arrives while its multiply-adds hold the
+// FP64 pipe (64 heat cubes 197 us, with one stage and 20 warps 203).  In fixed point one stage and 20 warps, whose
+// integer chains need the others (152 us, with two stages and 12 warps 174; a quarter in FP64 135 and 158).
+template <bool kFixed>
+struct ApplyShape {
+  static constexpr int kStages = kFixed ? 1 : 2, kCtas = kFixed ? 5 : 3;
+};
+
+template <int kStages>
+struct ApplyWarp {
+  double T[kStages][32 * kStride];                 // stages of a tile (column c, row r: c kStride + r)
+  double pJ[32], pI[32];                           // lambda blocks J and I
+  __align__(16) int2 lJ[32];                       // their limbs
+  __align__(16) int2 lI[32];
+};
+
+// q += sum of the tiles' products.  The tiles in storage order are cut into one run per warp
+// (runs of equal length: the (subdomain, row block) pairs hold 1 .. nt tiles, and a CTA for each left SMs
+// waiting), the tiles copied asynchronously; the row block's sum stays in
+// registers over its run, the columns' sums are added tile by tile.
+// kFixed: of every four tiles of a row block fp64_quarters (0..4) are multiplied in FP64 (FP64 pipe) and the
+// rest in fixed point (integer pipes), so that both pipes work at once; else all in FP64.
+// Bound by the FP64 pipe (64 multiply-adds of 16 cycles a tile and SM: 173 us for 64 heat cubes), in fixed point by
+// integer issue.  64 heat cubes (437 MB): FP64 246 -> 197 us, fixed 177 -> 152, a quarter in FP64 168 -> 135 (3.2 TB/s);
+// 710 tiles: 31 -> 15 us.
+template <bool kFixed>
+__global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
+    apply_tiles_kernel(const PlanPtrs P, int64_t n_tasks, int64_t n_tiles, const double *__restrict__ F,
+                       const double *__restrict__ lam, double *__restrict__ q, int fp64_quarters) {
+  extern __shared__ __align__(16) unsigned char apply_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kStages = ApplyShape<kFixed>::kStages;
+  ApplyWarp<kStages> &sm = reinterpret_cast<ApplyWarp<kStages> *>(apply_smem)[warp];
+  const int64_t nw = (int64_t)gridDim.x * kApplyWarps, w = (int64_t)blockIdx.x * kApplyWarps + warp;
+  const int64_t t0 = n_tiles * w / nw, t1 = n_tiles * (w + 1) / nw;
+  if (t0 >= t1) return;
+  const bool wide = (reinterpret_cast<uintptr_t>(F) & 15) == 0;   // F is 8-byte aligned, 16 is usual
+  auto fetch = [&](int64_t t, int buf) {
+    if (!wide) {
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sm.T[buf][lane]);
 #pragma unroll 8
-    for (int c = 0; c < 32; ++c) {
-      const double v = Tg[c * 32 + lane];
-      Ts[warp][c][lane] = v;
-      em = max(em, exp_field(v));
+      for (int c = 0; c < 32; ++c)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst + (uint32_t)(c * kStride * 8)),
+                     "l"(F + t * 1024 + c * 32 + lane)
+                     : "memory");
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      return;
     }
-    const uint32_t exT = __reduce_max_sync(kFull, em);
-    const int colJ = J * kTile + lane;
-    const double pJ = colJ < sd.m ? lam[map[colJ]] : 0.0;
-    if (((J >> 2) + J) % 4 < fp64_quarters) {     // this tile on the FP64 pipe (uniform across the warp)
-      __syncwarp();
-#pragma unroll 8
-      for (int c = 0; c < 32; ++c) y = fma(Ts[warp][c][lane], __shfl_sync(kFull, pJ, c), y);
-      if (J < I) {
-        double z = 0.0;
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) z = fma(Ts[warp][lane][r], __shfl_sync(kFull, pI, r), z);
-        if (colJ < sd.m) atomicAdd(q + map[colJ], z);
-      }
-      __syncwarp();
-      continue;
-    }
-    const uint32_t exJ = __reduce_max_sync(kFull, exp_field(pJ));
-    if (exT == 0) continue;                        // an all-zero tile adds nothing (uniform)
-    // each lane converts the entries it staged, in place
-#pragma unroll 8
-    for (int c = 0; c < 32; ++c) Tl[c * 33 + lane] = fixed_limbs(Ts[warp][c][lane], exT);
-    LJ[warp][lane] = fixed_limbs(pJ, exJ);
-    __syncwarp();
-    // rows: lane = row i of the tile, sum over its columns c
-    if (exJ != 0) {
-      long long d0 = 0, d1 = 0, d2 = 0;
-#pragma unroll 8
-      for (int c = 0; c < 32; ++c) mac(d0, d1, d2, Tl[c * 33 + lane], LJ[warp][c]);
-      y += combine(d0, d1, d2, (int)exT + (int)exJ - 2094);
-    }
-    // columns (off-diagonal tiles): lane = column j, sum over the tile's rows r
-    if (J < I && exI != 0) {
-      long long d0 = 0, d1 = 0, d2 = 0;
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) mac(d0, d1, d2, Tl[lane * 33 + r], LI[warp][r]);
-      if (colJ < sd.m) atomicAdd(q + map[colJ], combine(d0, d1, d2, (int)exT + (int)exI - 2094));
-    }
-    __syncwarp();
-  }
-  red[warp][lane] = y;
-  __syncthreads();
-  if (warp == 0) {
-    double s = 0.0;
+    const double *src = F + t * 1024 + 2 * lane;   // 16 bytes a lane: two columns to an instruction
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sm.T[buf][(lane >> 4) * kStride + 2 * (lane & 15)]);
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w][lane];
-    if (rowI < sd.m) atomicAdd(q + map[rowI], s);
+    for (int c = 0; c < 32; c += 2)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + (uint32_t)(c * kStride * 8)), "l"(src + c * 32)
+                   : "memory");
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  fetch(t0, 0);
+  TileCursor cur = tile_at(P, n_tasks, t0);
+  const int32_t *map = P.lambda + P.subs[cur.sub].col_off;
+  int row = 0, qI = -1;
+  uint32_t exI = 0;
+  auto load_I = [&]() {                            // lambda block I of the cursor's row block
+    row = cur.I * kTile + lane;
+    qI = row < cur.m ? map[row] : -1;
+    const double p = qI >= 0 ? lam[qI] : 0.0;
+    __syncwarp();
+    sm.pI[lane] = p;
+    if (kFixed) {
+      exI = __reduce_max_sync(kFull, exp_field(p));
+      sm.lI[lane] = fixed_limbs(p, exI);
+    }
+  };
+  load_I();
+  double y = 0.0;
+  for (int64_t t = t0; t < t1; ++t) {
+    const int buf = (int)(t - t0) % kStages;
+    const int J = cur.J, colJ = J * kTile + lane;
+    const bool offdiag = J < cur.I;
+    const int qJ = colJ < cur.m ? map[colJ] : -1;
+    const double p = qJ >= 0 ? lam[qJ] : 0.0;
+    if (kStages > 1 && t + 1 < t1) {
+      fetch(t + 1, (buf + 1) % kStages);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+    sm.pJ[lane] = p;
+    __syncwarp();
+    double *T = sm.T[buf];
+    if (!kFixed || J % 4 < fp64_quarters) {        // uniform across the warp
+      double y0 = 0.0, y1 = 0.0;                   // the tile's own sum, two chains
+#pragma unroll 8
+      for (int c = 0; c < 32; c += 2) {
+        const double2 l = *reinterpret_cast<const double2 *>(&sm.pJ[c]);
+        y0 = fma(T[c * kStride + lane], l.x, y0);
+        y1 = fma(T[(c + 1) * kStride + lane], l.y, y1);
+      }
+      y += y0 + y1;
+      if (offdiag) {
+        double z0 = 0.0, z1 = 0.0;
+#pragma unroll 8
+        for (int r = 0; r < 32; r += 2) {
+          const double2 v = *reinterpret_cast<const double2 *>(&T[lane * kStride + r]);
+          const double2 l = *reinterpret_cast<const double2 *>(&sm.pI[r]);
+          z0 = fma(v.x, l.x, z0);
+          z1 = fma(v.y, l.y, z1);
+        }
+        if (qJ >= 0) atomicAdd(q + qJ, z0 + z1);
+      }
+    } else if constexpr (kFixed) {
+      uint32_t em = 0;
+#pragma unroll 8
+      for (int c = 0; c < 32; ++c) em = max(em, exp_field(T[c * kStride + lane]));
+      const uint32_t exT = __reduce_max_sync(kFull, em);
+      const uint32_t exJ = __reduce_max_sync(kFull, exp_field(p));
+      if (exT != 0) {                              // an all-zero tile adds nothing (uniform)
+        int2 *Tl = reinterpret_cast<int2 *>(T);    // each lane converts its row, in place
+#pragma unroll 8
+        for (int c = 0; c < 32; ++c) Tl[c * kStride + lane] = fixed_limbs(T[c * kStride + lane], exT);
+        sm.lJ[lane] = fixed_limbs(p, exJ);
+        __syncwarp();
+        if (exJ != 0) {
+          long long d0 = 0, d1 = 0, d2 = 0, e0 = 0, e1 = 0, e2 = 0;   // two chains each
+#pragma unroll 8
+          for (int c = 0; c < 32; c += 2) {
+            mac(d0, d1, d2, Tl[c * kStride + lane], sm.lJ[c]);
+            mac(e0, e1, e2, Tl[(c + 1) * kStride + lane], sm.lJ[c + 1]);
+          }
+          y += combine(d0 + e0, d1 + e1, d2 + e2, (int)exT + (int)exJ - 2094);
+        }
+        if (offdiag && exI != 0) {
+          long long d0 = 0, d1 = 0, d2 = 0, e0 = 0, e1 = 0, e2 = 0;
+#pragma unroll 8
+          for (int r = 0; r < 32; r += 2) {
+            const int4 v = *reinterpret_cast<const int4 *>(&Tl[lane * kStride + r]);
+            const int4 l = *reinterpret_cast<const int4 *>(&sm.lI[r]);
+            mac(d0, d1, d2, make_int2(v.x, v.y), make_int2(l.x, l.y));
+            mac(e0, e1, e2, make_int2(v.z, v.w), make_int2(l.z, l.w));
+          }
+          if (qJ >= 0) atomicAdd(q + qJ, combine(d0 + e0, d1 + e1, d2 + e2, (int)exT + (int)exI - 2094));
+        }
+      }
+    }
+    __syncwarp();                                  // the next copies overwrite this stage
+    if (t + 1 < t1) {
+      if (kStages == 1) fetch(t + 1, 0);
+      const int sub = cur.sub;
+      cur.next(P);
+      if (cur.J == 0) {                            // the row block is complete
+        if (qI >= 0) atomicAdd(q + qI, y);
+        y = 0.0;
+        if (cur.sub != sub) map = P.lambda + P.subs[cur.sub].col_off;
+        load_I();
+      }
+    }
   }
+  if (qI >= 0) atomicAdd(q + qI, y);
+}
+
+// q += the product, launched over all tiles
+template <bool kFixed>
+cudaError_t launch_tiles(const sc_ctx &c, const double *F, const double *lam, double *q, int fp64_quarters, cudaStream_t st) {
+  const int64_t nt = c.sizes.F_doubles / 1024;
+  if (nt == 0) return cudaSuccess;
+  constexpr int smem = (int)sizeof(ApplyWarp<ApplyShape<kFixed>::kStages>) * kApplyWarps;
+  cudaError_t e = cudaFuncSetAttribute(apply_tiles_kernel<kFixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t grid = std::min<int64_t>((int64_t)kGridSMs * ApplyShape<kFixed>::kCtas, (nt + kApplyWarps - 1) / kApplyWarps);
+  apply_tiles_kernel<kFixed><<<(unsigned)grid, 32 * kApplyWarps, smem, st>>>(c.ptrs(), c.n_apply, nt, F, lam, q,
+                                                                           fp64_quarters);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -159,20 +256,16 @@ sc_status apply_split(sc_ctx *ctx, const double *F_dev, const double *lambda_dev
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   if (ctx->n_dual > 0) e = cudaMemsetAsync(q_dev, 0, sizeof(double) * (size_t)ctx->n_dual, st);
-  // the largest shared-memory carve-out, so that six CTAs (37 KB each) fit an SM
-  if (e == cudaSuccess && ctx->n_apply > 0)
-    e = cudaFuncSetAttribute(apply_fixed_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess && ctx->n_apply > 0) {
-    apply_fixed_kernel<<<(unsigned)ctx->n_apply, kThreads, 0, st>>>(ctx->ptrs(), F_dev, lambda_dev, q_dev,
-                                                                     fp64_quarters);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess) e = launch_tiles<true>(*ctx, F_dev, lambda_dev, q_dev, fp64_quarters, st);
   if (e != cudaSuccess) return fail(ctx, SC_ERR_CUDA, std::string(who) + ": " + cudaGetErrorString(e));
   return SC_OK;
 }
 
 }  // namespace
+
+int sc::launch_apply(const sc_ctx &c, const double *F, const double *lam, double *q, void *stream) {
+  return (int)launch_tiles<false>(c, F, lam, q, 4, static_cast<cudaStream_t>(stream));
+}
 
 extern "C" sc_status sc_apply_fixed(sc_ctx *ctx, const double *F_dev, const double *lambda_dev, double *q_dev,
                                     void *stream) {

@@ -18,8 +18,6 @@
 //                    (paper Sec. 3.3), summed over the supernodes active on
 //                    both chunks; the epilogue writes it straight into the
 //                    user's column order (the final back-permutation).
-//   apply_kernel  -- q += scatter(F_i gather(lambda)) reading each stored
-//                    lower tile once and using it for both triangles.
 //   export_kernel -- tile-packed F_i -> dense full column-major matrix.
 //
 // FP64 on GB300 is a narrow pipe (about 1.2 TFLOP/s for the whole GPU), so
@@ -330,46 +328,6 @@ __global__ void __launch_bounds__(kThreads, 6) syrk_kernel(const PlanPtrs P, con
   }
 }
 
-__global__ void __launch_bounds__(kThreads) apply_kernel(const PlanPtrs P, const double *__restrict__ F,
-                                                         const double *__restrict__ lam,
-                                                         double *__restrict__ q) {
-  __shared__ double Ts[kThreads / 32][32][33];
-  __shared__ double red[kThreads / 32][32];
-  const ApplyTask t = P.apply_tasks[blockIdx.x];
-  const SubDev sd = P.subs[t.sub];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int32_t *map = P.lambda + sd.col_off;
-  const int I = t.I;
-  const int rowI = I * kTile + lane;
-  const double pI = rowI < sd.m ? lam[map[rowI]] : 0.0;
-  double y = 0.0;
-  for (int J = warp; J <= I; J += kThreads / 32) {
-    const double *Tg = F + sd.F_off + ((int64_t)I * (I + 1) / 2 + J) * (kTile * kTile);
-#pragma unroll 8
-    for (int c = 0; c < 32; ++c) Ts[warp][c][lane] = Tg[c * 32 + lane];
-    __syncwarp();
-    const int colJ = J * kTile + lane;
-    const double pJ = colJ < sd.m ? lam[map[colJ]] : 0.0;
-#pragma unroll 8
-    for (int c = 0; c < 32; ++c) y = fma(Ts[warp][c][lane], __shfl_sync(0xffffffffu, pJ, c), y);
-    if (J < I) {
-      double z = 0.0;
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) z = fma(Ts[warp][lane][r], __shfl_sync(0xffffffffu, pI, r), z);
-      if (colJ < sd.m) atomicAdd(q + map[colJ], z);
-    }
-    __syncwarp();
-  }
-  red[warp][lane] = y;
-  __syncthreads();
-  if (warp == 0) {
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w][lane];
-    if (rowI < sd.m) atomicAdd(q + map[rowI], s);
-  }
-}
-
 __global__ void export_kernel(const SubDev *__restrict__ subs, int32_t i, const double *__restrict__ F,
                               double *__restrict__ dst, int32_t ld) {
   const SubDev sd = subs[i];
@@ -487,11 +445,6 @@ int launch_group_syrk(const sc_ctx &c, int w, int v, const double *Y, void *ws, 
   if (e) return e;
   if (v & kVarTile) return launch_syrk_tc(c, S, G.syrk[v][0], G.syrk[v][1], ws, F, stream);
   return launch_syrk_split(c, S, G.syrk[v][0], G.syrk[v][1], ws, F, stream);
-}
-
-int launch_apply(const sc_ctx &c, const double *F, const double *lam, double *q, void *stream) {
-  if (c.n_apply > 0) apply_kernel<<<(unsigned)c.n_apply, kThreads, 0, S(stream)>>>(c.ptrs(), F, lam, q);
-  return (int)cudaGetLastError();
 }
 
 int launch_export(const sc_ctx &c, const double *F, int32_t i, double *dst, int32_t ld, void *stream) {
