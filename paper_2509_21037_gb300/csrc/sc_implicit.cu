@@ -942,21 +942,40 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\
 
 // Of a group that works on one supernode of more than 32 columns: per stage the diagonal block
 // and its neighbour (forward: the rows below; backward: the columns before), the solved
-// block and the block's sums from this CTA.
+// block and the block's sums.
 struct TierStage {
   double D[2][32][33], N[2][32][33];
   double ys[2][32], sum[2][32];
 };
 
-// Supernodes of more than 32 columns by a group of warps of one CTA, one barrier per 32-column block.  The chain is the triangles: the group's first
-// warp solves block b and, in the same steps, forms the next 32 rows' update (forward) or the block
-// before's sums (backward), so that its next triangle waits for nobody; meanwhile the other warps
-// update the remaining rows with the block before (forward), or sum them for the block before's
-// columns (backward), and copy the next step's blocks into shared memory.  Bound by the chain and the
-// FP64 pipe it shares: a warp alone on its SM takes a step of the chain (a multiplication and two multiply-adds
-// of 64 cycles each, two shuffles) in 241 cycles, one beside 15 others with multiply-adds in 1495.  588
-// columns: 128 us forward, 143 backward (a cluster of eight SMs whose first has the chain to itself:
-// 106 and 147, and slower on the levels below).
+// Supernodes of more than 32 columns by a group of warps of one CTA, one barrier per 32-column block.  The
+// chain is the triangles: the group's first warp solves block b and, in the same steps, forms the next 32
+// rows' update (forward) or the block before's sums (backward), so that its next triangle waits for nobody;
+// meanwhile other warps update the remaining rows with the block before (forward), or sum them for the
+// block before's columns (backward), and copy the next step's blocks into shared memory.  Bound by the chain
+// and the FP64 pipe it shares: a warp alone on its SM takes a step of the chain (a multiplication and two
+// multiply-adds of 64 cycles each, two shuffles) in 241 cycles, one beside 15 others with multiply-adds in
+// 1495.  588 columns with every other warp helping: 128 us forward, 143 backward (a cluster of eight SMs whose
+// first has the chain to itself: 106 and 147, and slower on the levels below).  A triangle scaled by its
+// reciprocal diagonal takes the multiplication out of the chain, but rounds every entry once more: products
+// 1 to 6 % faster or slower, their error a tenth larger.
+
+// The warps that update or sum rows beside the chain: index hw of nh, -1 for none.  Warps w, w + 4, .. share a
+// sub-partition and its FP64 pipe, so in a group of eight or more the first warp's stays the chain's.  Whole
+// products, with every other warp helping and so: 16 mixed subdomains 1353 -> 1284 us, four elasticity cubes of
+// 12^3 to 14^3 nodes 1444 -> 1377, 64 heat cubes of 17^3 835 -> 824; none slower.  A smaller group would lose a
+// third or more of its helpers.
+__device__ __forceinline__ void helper_of(const Group &g, int &hw, int &nh) {
+  if (g.nw >= 8) {
+    const int q = g.gw >> 2, r = g.gw & 3;
+    hw = r ? 3 * q + r - 1 : -1;
+    nh = 3 * (g.nw >> 2) + max((g.nw & 3) - 1, 0);
+    return;
+  }
+  hw = g.gw - 1;
+  nh = g.nw - 1;
+}
+
 __device__ void forward_big(const Group &g, const ISn &sn, const double *__restrict__ Lv,
                             const int32_t *__restrict__ rows, double *x, int64_t rd_off, TierStage &st) {
   const int ns = sn.ns, nr = ns + sn.rs, nb = (ns + 31) >> 5, lane = g.lane;
@@ -972,6 +991,8 @@ __device__ void forward_big(const Group &g, const ISn &sn, const double *__restr
   stage(0, g.gw, g.nw);
   stage_wait();
   g.sync_cta();
+  int hw, nh;
+  helper_of(g, hw, nh);
   double accn = 0.0;                  // the first warp's: update of rows 32 b + lane by block b - 1
   for (int b = 0; b < nb; ++b) {
     const int w = min(32, ns - 32 * b);
@@ -995,8 +1016,8 @@ __device__ void forward_big(const Group &g, const ISn &sn, const double *__restr
       st.ys[b & 1][lane] = own ? xi : 0.0;
     } else {
       if (b + 1 < nb) stage(b + 1, g.gw - 1, g.nw - 1);
-      if (b > 0)
-        for (int t0 = 32 * (b + g.gw); t0 < nr; t0 += 32 * (g.nw - 1))
+      if (b > 0 && hw >= 0)
+        for (int t0 = 32 * (b + 1 + hw); t0 < nr; t0 += 32 * nh)
           forward_panel_chunk<false>(L, R, ns, nr, 32 * (b - 1), 32, t0, st.ys[(b - 1) & 1], xs, x, lane);
       stage_wait();
     }
@@ -1022,16 +1043,16 @@ __device__ void backward_big(const Group &g, const ISn &sn, const double *__rest
     if (b > 0) stage_block(st.N[b & 1], L, nr, 32 * (b - 1), 32, 32 * b, w, gw, nw, lane);
   };
   // st.sum[b & 1] = the sums over rows t_lo, .. of L(t, column) z_t for block b's columns; the
-  // 32-row chunks are shared by the group's warps from first_warp on
-  auto sums = [&](int b, int t_lo, int first_warp) {
-    const int kb = 32 * b, w = min(32, ns - kb), idx = g.gw - first_warp, cnt = g.nw - first_warp;
+  // calling warp is number idx of the cnt that share the 32-row chunks
+  auto sums = [&](int b, int t_lo, int idx, int cnt) {
+    const int kb = 32 * b, w = min(32, ns - kb);
     if (t_lo + 32 * idx < nr) {
       double acc[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) acc[k] = 0.0;
       for (int t0 = t_lo + 32 * idx; t0 < nr; t0 += 32 * cnt)
         backward_panel_chunk<false>(L, R, ns, nr, kb, w, t0, xs, x, acc, lane);
-      red[g.warp][lane] = transpose_reduce_w(acc, lane, w);
+      red[g.warp - g.gw + idx][lane] = transpose_reduce_w(acc, lane, w);
     }
     asm volatile("bar.sync %0, %1;\n" ::"r"(8 + g.slot), "r"(32 * cnt) : "memory");
     if (idx == 0) {
@@ -1040,13 +1061,15 @@ __device__ void backward_big(const Group &g, const ISn &sn, const double *__rest
       for (int v = 0; v < have; v += 4)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (v + j < have) s[j] += red[g.warp + v + j][lane];
+          if (v + j < have) s[j] += red[g.warp - g.gw + v + j][lane];
       st.sum[b & 1][lane] = (s[0] + s[1]) + (s[2] + s[3]);
     }
   };
+  int hw, nh;
+  helper_of(g, hw, nh);
   g.sync_cta();
   stage(nb - 1, g.gw, g.nw);
-  sums(nb - 1, ns, 0);
+  sums(nb - 1, ns, g.gw, g.nw);
   stage_wait();
   g.sync_cta();
   double accp = 0.0;
@@ -1069,7 +1092,7 @@ __device__ void backward_big(const Group &g, const ISn &sn, const double *__rest
       if (own) xs[32 * b + lane] = rhs;
     } else if (b > 0) {
       stage(b - 1, g.gw - 1, g.nw - 1);
-      sums(b - 1, 32 * b + w, 1);
+      if (hw >= 0) sums(b - 1, 32 * b + w, hw, nh);
       stage_wait();
     }
     g.sync_cta();
