@@ -69,19 +69,23 @@ constexpr int kStride = 34;                        // doubles between a tile's c
 constexpr int kApplyWarps = 4;                     // warps per CTA
 
 // In FP64 two stages per warp and 12 warps per SM: a warp's next tile arrives while its multiply-adds hold the
-// FP64 pipe (64 heat cubes 197 us, with one stage and 20 warps 203).  In fixed point one stage and 20 warps, whose
-// integer chains need the others (152 us, with two stages and 12 warps 174; a quarter in FP64 135 and 158).
+// FP64 pipe (64 heat cubes 197 us, with one stage and 20 warps 203).  In fixed point one stage and 24 warps, whose
+// integer chains need the others (64 heat cubes 146 us and a quarter in FP64 128; 20 warps 150 and 133; two stages and
+// 12 warps 174 and 158); the limbs of lambda block J lie over the block itself so that six CTAs fit an SM.
 template <bool kFixed>
 struct ApplyShape {
-  static constexpr int kStages = kFixed ? 1 : 2, kCtas = kFixed ? 5 : 3;
+  static constexpr int kStages = kFixed ? 1 : 2, kCtas = kFixed ? 6 : 3;
 };
 
 template <int kStages>
 struct ApplyWarp {
   double T[kStages][32 * kStride];                 // stages of a tile (column c, row r: c kStride + r)
-  double pJ[32], pI[32];                           // lambda blocks J and I
-  __align__(16) int2 lJ[32];                       // their limbs
-  __align__(16) int2 lI[32];
+  union {                                          // lambda block J, in fixed point its limbs
+    __align__(16) double pJ[32];
+    __align__(16) int2 lJ[32];
+  };
+  double pI[32];                                   // lambda block I
+  __align__(16) int2 lI[32];                       // and its limbs
 };
 
 // q += sum of the tiles' products.  The tiles in storage order are cut into one run per warp
@@ -91,8 +95,9 @@ struct ApplyWarp {
 // kFixed: of every four tiles of a row block fp64_quarters (0..4) are multiplied in FP64 (FP64 pipe) and the
 // rest in fixed point (integer pipes), so that both pipes work at once; else all in FP64.
 // Bound by the FP64 pipe (64 multiply-adds of 16 cycles a tile and SM: 173 us for 64 heat cubes), in fixed point by
-// integer issue.  64 heat cubes (437 MB): FP64 246 -> 197 us, fixed 177 -> 152, a quarter in FP64 168 -> 135 (3.2 TB/s);
-// 710 tiles: 31 -> 15 us.
+// integer issue.  64 heat cubes (437 MB): FP64 246 -> 197 us, fixed 177 -> 146, a quarter in FP64 168 -> 128 (3.4 TB/s);
+// 710 tiles: 31 -> 15 us; 657,000 tiles, where the ends of the runs don't count: FP64 2383 -> 2295, fixed 1576 -> 1592,
+// a quarter in FP64 1480 -> 1357.
 template <bool kFixed>
 __global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
     apply_tiles_kernel(const PlanPtrs P, int64_t n_tasks, int64_t n_tiles, const double *__restrict__ F,
