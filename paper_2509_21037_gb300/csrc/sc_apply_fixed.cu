@@ -95,9 +95,9 @@ struct ApplyWarp {
 // kFixed: of every four tiles of a row block fp64_quarters (0..4) are multiplied in FP64 (FP64 pipe) and the
 // rest in fixed point (integer pipes), so that both pipes work at once; else all in FP64.
 // Bound by the FP64 pipe (64 multiply-adds of 16 cycles a tile and SM: 173 us for 64 heat cubes), in fixed point by
-// integer issue.  64 heat cubes (437 MB): FP64 246 -> 197 us, fixed 177 -> 146, a quarter in FP64 168 -> 128 (3.4 TB/s);
-// 710 tiles: 31 -> 15 us; 657,000 tiles, where the ends of the runs don't count: FP64 2383 -> 2295, fixed 1576 -> 1592,
-// a quarter in FP64 1480 -> 1357.
+// integer issue.  64 heat cubes (437 MB): FP64 246 -> 197 us, fixed 177 -> 144, a quarter in FP64 168 -> 127 (3.4 TB/s);
+// 710 tiles: 31 -> 15 us; 657,000 tiles, where the ends of the runs don't count: FP64 2383 -> 2295, fixed 1576 both,
+// a quarter in FP64 1480 -> 1347.
 template <bool kFixed>
 __global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
     apply_tiles_kernel(const PlanPtrs P, int64_t n_tasks, int64_t n_tiles, const double *__restrict__ F,
@@ -183,10 +183,10 @@ __global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
         if (qJ >= 0) atomicAdd(q + qJ, z0 + z1);
       }
     } else if constexpr (kFixed) {
-      uint32_t em = 0;
+      uint32_t em = 0;                             // the largest high word holds the largest exponent
 #pragma unroll 8
-      for (int c = 0; c < 32; ++c) em = max(em, exp_field(T[c * kStride + lane]));
-      const uint32_t exT = __reduce_max_sync(kFull, em);
+      for (int c = 0; c < 32; ++c) em = max(em, (uint32_t)__double2hiint(T[c * kStride + lane]) & 0x7FFFFFFFu);
+      const uint32_t exT = __reduce_max_sync(kFull, em) >> 20;
       const uint32_t exJ = __reduce_max_sync(kFull, exp_field(p));
       if (exT != 0) {                              // an all-zero tile adds nothing (uniform)
         int2 *Tl = reinterpret_cast<int2 *>(T);    // each lane converts its row, in place
@@ -198,8 +198,9 @@ __global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
           long long d0 = 0, d1 = 0, d2 = 0, e0 = 0, e1 = 0, e2 = 0;   // two chains each
 #pragma unroll 8
           for (int c = 0; c < 32; c += 2) {
-            mac(d0, d1, d2, Tl[c * kStride + lane], sm.lJ[c]);
-            mac(e0, e1, e2, Tl[(c + 1) * kStride + lane], sm.lJ[c + 1]);
+            const int4 l = *reinterpret_cast<const int4 *>(&sm.lJ[c]);
+            mac(d0, d1, d2, Tl[c * kStride + lane], make_int2(l.x, l.y));
+            mac(e0, e1, e2, Tl[(c + 1) * kStride + lane], make_int2(l.z, l.w));
           }
           y += combine(d0 + e0, d1 + e1, d2 + e2, (int)exT + (int)exJ - 2094);
         }
