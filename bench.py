@@ -163,14 +163,18 @@ class ClockSampler:
                 "samples": len(sm), "reasons": sorted(reasons)}
 
 
-# the source file of each profiled kernel
-_KERNEL_SOURCE = {"apply_digits_kernel": "sc_apply_digits.cu", "apply_fixed_kernel": "sc_apply_fixed.cu",
-                  "implicit_kernel": "sc_implicit.cu"}
+# the source files of each profiled kernel
+_KERNEL_SOURCE = {"syrk_kernel": ("sc_kernels.cu",), "trsm_kernel": ("sc_kernels.cu", "sc_trsm.cuh"),
+                  "apply_tiles_kernel": ("sc_apply_fixed.cu", "sc_tiles.cuh"),
+                  "apply_digits_kernel": ("sc_apply_digits.cu", "sc_tiles.cuh"),
+                  "tier_kernel": ("sc_implicit.cu",)}
 
 
 def _kernel_source_hash(kernel: str = "syrk_kernel"):
-    src = os.path.join(ROOT, "paper_2509_21037_gb300", "csrc", _KERNEL_SOURCE.get(kernel, "sc_kernels.cu"))
-    return hashlib.sha256(open(src, "rb").read()).hexdigest()
+    h = hashlib.sha256()
+    for src in _KERNEL_SOURCE[kernel]:
+        h.update(open(os.path.join(ROOT, "paper_2509_21037_gb300", "csrc", src), "rb").read())
+    return h.hexdigest()
 
 
 def _traffic_for(kernel: str):
@@ -692,7 +696,7 @@ def run_sc(args):
                          "iterations_vs_gpu_implicit_fixed_apply": t_asm / (t_gimpl - t_fixed) if t_gimpl > t_fixed else None},
         "sc_apply": apply_sec,
         "gpu_implicit_apply": gimpl,
-        "gpu_launches": args.steps * 5,
+        "gpu_launches": args.steps * 4,               # prep, TRSM, SYRK, apply
         "clocks": clocks.summary(),
     }
     if args.feti and rank == 0:

@@ -105,7 +105,8 @@ enum { SC_FP64 = 0, SC_SPLIT_BF16 = 1 };
  *            on the tensor cores as exact products of 8-bit digit planes of
  *            the FP64 operands (BF16 in, FP32 accumulate, integer and FP64
  *            combination), n_slices digits per operand; the diagonal-triangle
- *            solves and the accumulation into Y and F stay FP64.  The error
+ *            solves, the updates below diagonal blocks of at most four columns
+ *            and the accumulation into Y and F stay FP64.  The error
  *            is below about 2^(-8 n_slices) relative to the product of the
  *            operands' column bounds; n_slices = 7 keeps 56 bits.
  * n_slices: 3..7 for SC_SPLIT_BF16 (0 selects 7); ignored for SC_FP64.
@@ -123,10 +124,11 @@ enum { SC_FP64 = 0, SC_SPLIT_BF16 = 1 };
  *            waves run one after the other and reuse the same workspace (the
  *            paper's temporary memory pool, Sec. 3.1).  SC_ERR_OOM if one
  *            subdomain alone does not fit. */
-/* persistent: 0 (default) launches one CTA per FP64 TRSM / SYRK task and
- *            lets the hardware block scheduler hand them out; 1 launches as
- *            many CTAs as the GPU keeps resident, which pull task indices
- *            (largest first) from an atomic counter in the workspace status
+/* persistent: 0 (default) launches a CTA for every four parts of the FP64 TRSM
+ *            tasks (a warp each) and for every FP64 SYRK task or part of one,
+ *            and lets the hardware block scheduler hand them out; 1 launches as
+ *            many CTAs as the GPU keeps resident, which pull part indices
+ *            (largest task first) from an atomic counter in the workspace status
  *            area until the list is exhausted (a persistent work queue; no
  *            CTA waits on another). */
 /* tile:     SYRK output tile of the split-precision subdomains: SC_TILE_32
@@ -276,8 +278,8 @@ sc_status sc_apply_fixed(sc_ctx *ctx, const double *F_dev, const double *lambda_
                          void *stream);
 
 /* The same product with the stored tiles split between GB300's two
- * arithmetic paths so that both work at once: of every four tiles a warp
- * visits, fp64_quarters (0..4) are multiplied in FP64 on the FP64 pipe (as
+ * arithmetic paths so that both work at once: of every four tiles of a
+ * row block, fp64_quarters (0..4) are multiplied in FP64 on the FP64 pipe (as
  * sc_apply) and the rest in fixed point on the integer pipes (as
  * sc_apply_fixed); each row and tile is rounded once either way, so the
  * error bound is that of the two forms.  fp64_quarters = 0 is sc_apply_fixed.

@@ -115,13 +115,16 @@ sc_status sci_device_status(sci_ctx *ctx, const void *ws_dev, void *stream);
 /* Host copy of the plan tables (bytes >= plan_bytes), for inspection.  Layout:
  * a 256-byte header {uint32 magic 'SCIP', uint32 version 1, int32 nsub, pad,
  * int64 n_sn, n_levptr, n_rows, n_grow, n_gent, n_sent, n_items,
- * uint64 sec_off[8]} and eight 256-byte aligned sections: subdomains (48 B each, largest first:
- * int64 x_off; int32 n, sn_lo, sn_hi, lev_lo, n_lev, g_lo, g_hi, s_lo, s_hi,
- * pad), supernodes (32 B: int64 lval, rows_off; int32 c0, ns, rs, sub),
+ * uint64 sec_off[8], piece_off, int64 n_pieces} and nine 256-byte aligned
+ * sections: subdomains (64 B each, largest first: int64 x_off; int32 n, sn_lo,
+ * sn_hi, lev_lo, n_lev, g_lo, g_hi, s_lo, s_hi, and the pair form's n_lev_a,
+ * n_lev_b, s_mid1, s_mid2, pad), supernodes (32 B: int64 lval, rows_off; int32 c0, ns, rs, sub),
  * level boundaries (int32), pruned rows (int32), gather rows (int32 r, e_lo,
  * e_hi, pad), gather entries (int32 gj, sign), scatter entries (int32 r, gj,
  * sign, pad), cluster items (int32 kind, n, sub[8]; kind 0: sub[0] on the
- * whole cluster, kind 1: sub[r] on CTA r for r < n). */
+ * whole cluster, kind 1: sub[r] on CTA r for r < n),
+ * pieces of the tiered schedule (int32 sub, lev_lo, n_lev, s_lo, s_hi, pad; tier
+ * by tier: levels and scatter entries as in the subdomains). */
 sc_status sci_export_plan(const sci_ctx *ctx, void *dst, size_t bytes);
 
 const char *sci_last_error(const sci_ctx *ctx);
