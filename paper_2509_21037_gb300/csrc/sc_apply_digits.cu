@@ -247,6 +247,25 @@ __device__ __forceinline__ long long class_sum(const float (&d)[2][4], float c0,
   return k;
 }
 
+// Loads of lambda's digits, which the lambda kernel may still be writing when the product starts: volatile, so that
+// they stay behind griddepcontrol.wait.  Plain loads through a const __restrict__ pointer could be moved ahead of it or
+// take the read-only path, since that qualifier says that nobody writes there while the kernel runs.
+__device__ __forceinline__ uint4 load_written(const unsigned char *p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 load_written_float2(const unsigned char *p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0,%1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ int load_written_int(const unsigned char *p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar));
 }
@@ -293,8 +312,7 @@ __device__ __forceinline__ void fetch_lambda(uint32_t stage, uint32_t bar, const
 __global__ void __launch_bounds__(kPairs * 64, 1) apply_digits_kernel(const PlanPtrs P, int64_t n_tasks,
                                                                      int64_t n_tiles,
                                                                      const unsigned char *__restrict__ Fd,
-                                                                     const unsigned char *__restrict__ tab,
-                                                                     double *__restrict__ q,
+                                                                     unsigned char *tab, double *__restrict__ q,
                                                                      uint32_t *__restrict__ status,
                                                                      long long poll_limit) {
   extern __shared__ __align__(128) unsigned char dsm[];
@@ -346,11 +364,11 @@ __global__ void __launch_bounds__(kPairs * 64, 1) apply_digits_kernel(const Plan
   auto load_lamI = [&](int64_t task) {
     const unsigned char *ent = tab + task * kLamBytes;
 #pragma unroll
-    for (int k = 0; k < kDigitsF; ++k) bI[k] = reinterpret_cast<const uint4 *>(ent)[(g - k + 6) * 4 + t];
-    const float *cj = reinterpret_cast<const float *>(ent + kLamCjOff);
-    cI0 = cj[2 * t];
-    cI1 = cj[2 * t + 1];
-    eI = reinterpret_cast<const int *>(ent + kLamCjOff + 32)[0];
+    for (int k = 0; k < kDigitsF; ++k) bI[k] = load_written(ent + ((g - k + 6) * 4 + t) * 16);
+    const float2 cj = load_written_float2(ent + kLamCjOff + 8 * t);
+    cI0 = cj.x;
+    cI1 = cj.y;
+    eI = load_written_int(ent + kLamCjOff + 32);
   };
   if (half) load_lamI(cur.task);
   int s = 0;
@@ -527,7 +545,7 @@ extern "C" sc_status sc_apply_digits(sc_ctx *ctx, void *Fd_dev, const double *la
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         e = cudaLaunchKernelEx(&cfg, apply_digits_kernel, ctx->ptrs(), (int64_t)ctx->n_apply, nt,
-                               (const unsigned char *)Fd, (const unsigned char *)tab, q_dev,
+                               (const unsigned char *)Fd, tab, q_dev,
                                reinterpret_cast<uint32_t *>(Fd + status_offset(ctx)), limit);
       }
     }
