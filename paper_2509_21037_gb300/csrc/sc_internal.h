@@ -29,6 +29,10 @@ constexpr int kGridSMs = 152;   // SMs of a GB300: the round length of the TRSM 
 
 // bits of the workspace status word
 enum : uint32_t { kStatusNotSpd = 1u, kStatusTimeout = 2u };
+// The workspace begins with 256 bytes that start at zero: the status word, the persistent queues' words (at 64 and 128),
+// and, as 32-bit word 48, whether the split TRSM solves with its triangles as they are (prep_kernel).
+constexpr size_t kStatusBytes = 256;
+constexpr int kUnscaledWord = 48;
 
 // Per-subdomain kernel variant: 0 = FP64; S (3..7) = split precision with S
 // digits and 32x32 SYRK blocks (mma.sync); kVarTile | S = the same digits
@@ -228,7 +232,6 @@ int launch_groups(sc_ctx &c, int w, const double *Lv, const double *invd, void *
 int launch_lpack_split(const sc_ctx &c, int S, int64_t base, int64_t count, const double *Lv, void *ws, void *stream);
 int launch_trsm_split(const sc_ctx &c, int S, int cols, int64_t base, int64_t count, const double *Lv, const double *invd,
                       void *ws, double *Y, void *stream);
-int launch_colexp_reset(const sc_ctx &c, void *ws, void *stream);
 // balanced: digits in [-128, 128] against twice the column bound (the tcgen05 SYRK's planes)
 int launch_yslice_group(const sc_ctx &c, int S, int64_t base, int64_t count, const double *Y, void *ws,
                         void *stream, bool balanced);

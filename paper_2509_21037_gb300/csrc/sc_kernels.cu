@@ -37,13 +37,18 @@
 namespace sc {
 
 // One launch for what the stages need beforehand (two launches cost a small batch
-// 3 us of its 60).  CTAs below nprep: reciprocal diagonal.  The others, one per
+// 3 us of its 60).  CTAs below nprep: reciprocal diagonal.  The next, one per
 // subdomain: zero the entries of F beyond m (rows >= m of the last tile row and
-// columns >= m of the last diagonal tile).
+// columns >= m of the last diagonal tile).  The others, for split precision: zero the column bounds of Y and
+// look at the triangles, a warp to a (supernode, block).  Where an entry is so far from its column's diagonal (rows of L
+// that differ by hundreds of orders of magnitude) that FP64 may not hold their ratio in full, the
+// split TRSM must not divide its triangles by the diagonal.
 __global__ void __launch_bounds__(256) prep_kernel(const int64_t *__restrict__ lcp, const int32_t *__restrict__ active,
                                                    int64_t nact, int nprep, const double *__restrict__ Lv,
                                                    double *__restrict__ invd, uint32_t *__restrict__ status,
-                                                   const SubDev *__restrict__ subs, double *__restrict__ F) {
+                                                   const SubDev *__restrict__ subs, int nsub, double *__restrict__ F,
+                                                   const PlanPtrs P, int64_t nsblk, int *__restrict__ colexp,
+                                                   int64_t ncols) {
   if ((int)blockIdx.x < nprep) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nact; k += (int64_t)nprep * blockDim.x) {
       const int32_t g = active[k];
@@ -55,6 +60,27 @@ __global__ void __launch_bounds__(256) prep_kernel(const int64_t *__restrict__ l
         invd[g] = 1.0 / d;
       }
     }
+    return;
+  }
+  if ((int)blockIdx.x >= nprep + nsub) {
+    const int64_t cta = blockIdx.x - nprep - nsub, nt = (int64_t)(gridDim.x - nprep - nsub) * blockDim.x;
+    for (int64_t k = cta * blockDim.x + threadIdx.x; k < ncols; k += nt) colexp[k] = 0;
+    const int64_t item = cta * (blockDim.x / 32) + threadIdx.x / 32;
+    if (item >= nsblk) return;
+    const SnDev s = P.sns[P.sblk[2 * item]];
+    const int kb = 32 * P.sblk[2 * item + 1], kw = min(32, s.ns - kb), nr = s.ns + s.rs - kb, r = threadIdx.x & 31;
+    if (kw <= kDirect) return;
+    // high words; entry (t, q) of the triangle at q nr - q (q + 1) / 2 + t
+    const uint32_t *Lh = reinterpret_cast<const uint32_t *>(Lv + lcp[s.lcp_off + kb]) + 1;
+    bool out = false;
+#pragma unroll 8
+    for (int q = 0; q < kw; ++q) {
+      const int o = q * nr - q * (q + 1) / 2;
+      const uint32_t l = r > q && r < kw ? Lh[2 * (o + r)] : 0u, d = r > q && r < kw ? Lh[2 * (o + q)] : 0u;
+      const int e = (int)(l >> 20 & 0x7FFu), f = e - (int)(d >> 20 & 0x7FFu);
+      out |= (l << 1 != 0u) & ((e == 0) | (f < -1020) | (f > 1020));
+    }
+    if (out) status[kUnscaledWord] = 1u;
     return;
   }
   const SubDev sd = subs[blockIdx.x - nprep];
@@ -361,12 +387,16 @@ int launch_prep(const sc_ctx &c, const double *Lv, double *invd, uint32_t *statu
                 void *stream) {
   const PlanPtrs p = c.ptrs();
   const int nprep = (int)std::min<int64_t>((c.n_active_cols + 255) / 256, 152 * 16);
+  int64_t ncols = 0, ncheck = 0;
+  if (c.n_slices > 0) {
+    for (int32_t m : c.m) ncols += m;
+    ncheck = std::max<int64_t>((c.n_sblk + 7) / 8, ncols > 0);
+  }
   if (nprep + c.nsub > 0)
-    prep_kernel<<<(unsigned)(nprep + c.nsub), 256, 0, S(stream)>>>(p.lcp, p.active_cols, c.n_active_cols, nprep, Lv,
-                                                                   invd, status, p.subs, F);
-  int e = (int)cudaGetLastError();
-  if (!e && c.n_slices > 0) e = launch_colexp_reset(c, ws, stream);
-  return e;
+    prep_kernel<<<(unsigned)(nprep + c.nsub + ncheck), 256, 0, S(stream)>>>(
+        p.lcp, p.active_cols, c.n_active_cols, nprep, Lv, invd, status, p.subs, c.nsub, F, p, c.n_sblk,
+        reinterpret_cast<int *>(static_cast<uint8_t *>(ws) + c.ws.colexp_off), ncols);
+  return (int)cudaGetLastError();
 }
 
 template <int W>

@@ -46,10 +46,6 @@ namespace {
 
 using namespace digits;
 
-// TRSM blocks of at most kDirect columns update the rows below in FP64, a multiply-add per
-// column and entry of Y against the two operations that an entry costs after the digit products.
-constexpr int kDirect = 4;
-
 constexpr int kPad = 40;   // bf16 row stride of a digit plane (conflict-free fragment loads)
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -364,6 +360,51 @@ struct TrsmSplit {
   const int16_t *lexp;         // its rows' exponent bounds
   int64_t ld_rows;
   int *colexp;                 // exponent bounds of Y's columns (out)
+  const unsigned *unscaled;    // not 0: triangles are not divided by their diagonal (prep_kernel)
+};
+
+// A lane's fragments of the S digit planes of L, panel rows row (va) and row + 8 (vb), by 16-byte loads (kVector) or by words.
+template <int S, bool kVector>
+struct Fragments;
+template <int S>
+struct Fragments<S, false> {
+  uint32_t w[S][2][4];
+  __device__ __forceinline__ void load(const TrsmSplit &sp, int64_t row, bool va, bool vb, int tg) {
+#pragma unroll
+    for (int d = 0; d < S; ++d) {
+      const uint32_t *pw = reinterpret_cast<const uint32_t *>(sp.Ld + (int64_t)d * sp.ld_rows * 32) + row * 16 + 4 * tg;
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        w[d][ks][0] = va ? pw[2 * ks] : 0u;
+        w[d][ks][1] = vb ? pw[128 + 2 * ks] : 0u;
+        w[d][ks][2] = va ? pw[2 * ks + 1] : 0u;
+        w[d][ks][3] = vb ? pw[128 + 2 * ks + 1] : 0u;
+      }
+    }
+  }
+  // c += (the rows' plane d) (the column of X's digits at px)
+  __device__ __forceinline__ void mma(float (&c)[4], int d, const __nv_bfloat16 *px) const {
+    mma_bf16(c, w[d][0], ld_pair(px), ld_pair(px + 8));
+    mma_bf16(c, w[d][1], ld_pair(px + 16), ld_pair(px + 24));
+  }
+};
+template <int S>
+struct Fragments<S, true> {
+  uint4 a[S], b[S];
+  __device__ __forceinline__ void load(const TrsmSplit &sp, int64_t row, bool va, bool vb, int tg) {
+#pragma unroll
+    for (int d = 0; d < S; ++d) {
+      const uint4 *pl = reinterpret_cast<const uint4 *>(sp.Ld + (int64_t)d * sp.ld_rows * 32) + row * 4 + tg;
+      a[d] = va ? pl[0] : make_uint4(0u, 0u, 0u, 0u);
+      b[d] = vb ? pl[32] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  __device__ __forceinline__ void mma(float (&c)[4], int d, const __nv_bfloat16 *px) const {
+    const uint32_t w0[4] = {a[d].x, b[d].x, a[d].y, b[d].y};
+    const uint32_t w1[4] = {a[d].z, b[d].z, a[d].w, b[d].w};
+    mma_bf16(c, w0, ld_pair(px), ld_pair(px + 8));
+    mma_bf16(c, w1, ld_pair(px + 16), ld_pair(px + 24));
+  }
 };
 
 template <int C, int S>
@@ -465,13 +506,8 @@ __device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, 
             for (int r0 = 16 * warp; r0 < nb; r0 += 16 * (kThreads / 32)) {
               const int ra = r0 + g, rb = r0 + g + 8;
               const bool va = ra < nb, vb = rb < nb;
-              uint4 fa[S], fb[S];
-#pragma unroll
-              for (int d = 0; d < S; ++d) {
-                const uint4 *pl = reinterpret_cast<const uint4 *>(sp.Ld + (int64_t)d * sp.ld_rows * 32) + (base + ra) * 4 + tg;
-                fa[d] = va ? pl[0] : make_uint4(0u, 0u, 0u, 0u);
-                fb[d] = vb ? pl[32] : make_uint4(0u, 0u, 0u, 0u);
-              }
+              Fragments<S, true> fr;
+              fr.load(sp, base + ra, va, vb, tg);
               const int ea = va ? sp.lexp[base + ra] : 0, eb = vb ? sp.lexp[base + rb] : 0;
               double *ta = nullptr, *tb = nullptr;                 // this lane's two target rows
               if (va) ta = Y + colsh + (below + ra < s.ns ? s.y_off + (int64_t)(below + ra) * ws : rm[below + ra - s.ns]);
@@ -495,10 +531,7 @@ __device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, 
 #pragma unroll
                   for (int q = 0; q <= d; ++q) {
                     const __nv_bfloat16 *px = &sm.PX[d - q][8 * nt + g][2 * tg];
-                    const uint32_t a0[4] = {fa[q].x, fb[q].x, fa[q].y, fb[q].y};
-                    const uint32_t a1[4] = {fa[q].z, fb[q].z, fa[q].w, fb[q].w};
-                    mma_bf16(c, a0, ld_pair(px), ld_pair(px + 8));
-                    mma_bf16(c, a1, ld_pair(px + 16), ld_pair(px + 24));
+                    fr.mma(c, q, px);
                   }
 #pragma unroll
                   for (int r = 0; r < 4; ++r) gr[r].add(d, __float2int_rn(c[r]));
@@ -562,8 +595,199 @@ __global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(co
                                                               double *__restrict__ Y) {
   extern __shared__ __align__(16) unsigned char team_smem[];
   constexpr int kParts = kChunk / (4 * C);
+  if (*sp.unscaled) return;                                        // trsm_chunk_kernel takes the whole launch
   trsm_team<C, S>(P, P.trsm_tasks[blockIdx.x / kParts], blockIdx.x % kParts, Lv, invd, sp, Y,
                   *reinterpret_cast<TeamShared<C, S> *>(team_smem), threadIdx.x >> 5, threadIdx.x & 31);
+}
+
+// The same for a whole chunk of 32 columns by one CTA, the triangle shared by its warps 8 rows at a time.  Same operations in
+// the same order as trsm_team, so the same bits.  It runs behind trsm_split_kernel and takes the launch over
+// only where the triangles must not be divided by their diagonals: an empty launch otherwise.
+template <int S>
+__global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_chunk_kernel(const PlanPtrs P, const double *__restrict__ Lv,
+                                                                 const double *__restrict__ invd, const TrsmSplit sp,
+                                                                 double *__restrict__ Y) {
+  __shared__ double X[32][33];                              // the solved block: [row][live column]
+  __shared__ double T[32 * 31 / 2];
+  __shared__ __align__(16) __nv_bfloat16 PX[S][32][kPad];   // its digit planes: [digit][live column][row]
+  __shared__ int emax[32];
+  const bool unscaled = *sp.unscaled != 0;
+  if (!unscaled) return;
+  const TrsmTask t = P.trsm_tasks[blockIdx.x];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, tg = lane & 3;
+  const int c_hi = t.c_lo + t.w;
+  // the warp that solves: spread over the SM's sub-partitions across co-resident CTAs
+  const int tri = (int)((blockIdx.x * 2654435761u) >> 30);
+  int *colexp = sp.colexp + P.subs[t.sub].col_off;
+  for (int li = 0; li < t.list_len; ++li) {
+    const SnDev s = P.sns[P.trsm_list[t.list_off + li]];
+    const int a = max(s.jlo, t.c_lo), w = min(s.jhi, c_hi) - a, ws = s.jhi - s.jlo;
+    double *Ys = Y + s.y_off + (a - s.jlo);
+    for (int e = tid; e < s.ns * w; e += kThreads) {
+      const int r = e / w;
+      Ys[(int64_t)r * ws + e - r * w] = 0.0;
+    }
+  }
+  __syncthreads();
+  for (int e = t.seed_lo + tid; e < t.seed_hi; e += kThreads) Y[P.seeds[e].y_off] = P.seeds[e].value;
+  __syncthreads();
+
+  for (int li = 0; li < t.list_len; ++li) {
+    const SnDev s = P.sns[P.trsm_list[t.list_off + li]];
+    const int a = max(s.jlo, t.c_lo), b = min(s.jhi, c_hi), ws = s.jhi - s.jlo, colsh = a - s.jlo;
+    double *Ys = Y + s.y_off + colsh;
+    const double *id = invd + s.lcp_off;
+    const int64_t *rm = P.rmap + s.rmap_off;
+    const int nr = s.ns + s.rs;
+    const double *Lc = Lv + P.lcp[s.lcp_off];                // panel row t of column kb at Lc + t
+    for (int kb = 0, blk = 0; kb < s.ns; Lc += 32LL * (nr - kb) - 16 * 33, kb += 32, ++blk) {
+      const int kw = min(32, s.ns - kb), below = kb + kw, nb = nr - below;
+      const int wk = min(b, P.cuts[s.cut_off + blk]) - a;
+      if (wk <= 0) continue;
+      const int64_t base = s.ld_off + (int64_t)blk * nr - 16LL * blk * (blk + 1);
+      Fragments<S, false> fr;
+      auto load_fr = [&](int r0) { fr.load(sp, base + r0 + g, r0 + g < nb, r0 + g + 8 < nb, tg); };
+      const bool pre = warp != tri && kw > kDirect && 16 * warp < nb;
+      if (pre) load_fr(16 * warp);
+      for (int e = tid; e < kw * 32; e += kThreads) {
+        const int q = e >> 5, c = e & 31;
+        X[q][c] = c < wk ? Ys[(int64_t)(kb + q) * ws + c] : 0.0;
+      }
+      const bool scaled = kw > kDirect && !unscaled;
+#pragma unroll 4
+      for (int p = warp; p < kw; p += kThreads / 32)
+        if (lane > p && lane < kw) {
+          const double l = Lc[kb + lane + p * (nr - kb - 1) - p * (p - 1) / 2];
+          T[tri_at(lane, p)] = scaled ? l * id[kb + p] : l;
+        }
+      __syncthreads();
+      for (int p0 = 0; p0 < kw; p0 += 8) {
+        const int pe = min(p0 + 8, kw);
+        if (warp == tri && lane < wk) {
+          double x[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[i] = p0 + i < kw ? X[p0 + i][lane] : 0.0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (p0 + i >= kw) break;                         // uniform
+            if (!scaled) x[i] *= id[kb + p0 + i];
+#pragma unroll
+            for (int r = i + 1; r < 8; ++r)
+              if (p0 + r < kw) x[r] = fma(-T[tri_at(p0 + r, p0 + i)], x[i], x[r]);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (p0 + i < kw) X[p0 + i][lane] = x[i];
+        }
+        __syncthreads();
+        if (pe < kw) {                                       // then pe == p0 + 8
+          if (lane < wk) {
+            double x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = X[p0 + i][lane];
+            for (int r = pe + ((warp - tri) & 3); r < kw; r += kThreads / 32) {
+              double xr = X[r][lane];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) xr = fma(-T[tri_at(r, p0 + i)], x[i], xr);
+              X[r][lane] = xr;
+            }
+          }
+          __syncthreads();
+        }
+      }
+      if (warp == tri) {
+        int em = 0;
+        if (lane < wk)
+          for (int q = 0; q < kw; ++q) {
+            double v = X[q][lane];
+            if (scaled) X[q][lane] = v = v * id[kb + q];
+            Ys[(int64_t)(kb + q) * ws + lane] = v;
+            em = max(em, biased_exponent(v));
+          }
+        emax[lane] = em;
+        if (lane < wk && em) atomicMax(colexp + a + lane, em);
+      }
+      __syncthreads();
+      if (nb <= 0) continue;                                 // uniform
+      if (kw <= kDirect) {
+        // (row, live column) pairs numbered row by row and dealt to the threads in turn
+        const int dp = kThreads / wk, dc = kThreads - dp * wk;
+        int p = below + tid / wk, cl = tid - tid / wk * wk;
+        while (p < nr) {
+          double *tgt = (p < s.ns ? Ys + (int64_t)p * ws : Y + rm[p - s.ns] + colsh) + cl;
+          double acc = *tgt;
+          int o = p;
+          for (int q = 0; q < kw; ++q) {
+            acc = fma(-Lc[o], X[q][cl], acc);
+            o += nr - (kb + q) - 1;
+          }
+          *tgt = acc;
+          p += dp;
+          cl += dc;
+          if (cl >= wk) {
+            cl -= wk;
+            ++p;
+          }
+        }
+        __syncthreads();
+        continue;
+      }
+      for (int e = tid; e < 32 * 32; e += kThreads) {
+        const int q = e >> 5, c = e & 31;
+        const double v = (q < kw && c < wk) ? X[q][c] : 0.0;
+        const uint64_t m = fixed_point(v, emax[c]);
+#pragma unroll
+        for (int d = 0; d < S; ++d) PX[d][c][q] = digit_bf16(m, d, v < 0.0);
+      }
+      __syncthreads();
+      for (int r0 = 16 * warp; r0 < nb; r0 += 16 * (kThreads / 32)) {
+        const int ra = r0 + g, rb = r0 + g + 8;
+        const bool va = ra < nb, vb = rb < nb;
+        const int ea = va ? sp.lexp[base + ra] : 0, eb = vb ? sp.lexp[base + rb] : 0;
+        double *ta = nullptr, *tb = nullptr;                 // this lane's two target rows
+        if (va) ta = Y + colsh + (below + ra < s.ns ? s.y_off + (int64_t)(below + ra) * ws : rm[below + ra - s.ns]);
+        if (vb) tb = Y + colsh + (below + rb < s.ns ? s.y_off + (int64_t)(below + rb) * ws : rm[below + rb - s.ns]);
+        if (!(pre && r0 == 16 * warp)) load_fr(r0);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+          if (8 * nt >= wk) break;                           // uniform
+          // the targets' current values, loaded before the products so that
+          // their latency overlaps the MMAs
+          double yv[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const int col = 8 * nt + 2 * tg + (r & 1);
+            const double *p = (r & 2) ? tb : ta;
+            yv[r] = (p && col < wk) ? p[col] : 0.0;
+          }
+          Groups<S> gr[4];
+#pragma unroll
+          for (int d = 0; d < S; ++d) {
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int q = 0; q <= d; ++q) {
+              const __nv_bfloat16 *px = &PX[d - q][8 * nt + g][2 * tg];
+              fr.mma(c, q, px);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) gr[r].add(d, __float2int_rn(c[r]));
+          }
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const int col = 8 * nt + 2 * tg + (r & 1);
+            double *p = (r & 2) ? tb : ta;
+            if (p && col < wk) {
+              const int e = ((r & 2 ? eb : ea) - 1022) + (emax[col] - 1022) + Groups<S>::kBlockShift;
+              const double v = (double)gr[r].block_int();
+              p[col] = (e >= -1022 && e <= 1023) ? fma(-v, pow2i(e), yv[r]) : yv[r] - ldexp(v, e);
+            }
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
 }
 
 }  // namespace
@@ -607,23 +831,17 @@ int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t c
   uint8_t *w = static_cast<uint8_t *>(ws);
   const TrsmSplit sp{reinterpret_cast<const __nv_bfloat16 *>(w + c.ws.ld_off),
                      reinterpret_cast<const int16_t *>(w + c.ws.lexp_off), c.ws.ld_rows,
-                     reinterpret_cast<int *>(w + c.ws.colexp_off)};
+                     reinterpret_cast<int *>(w + c.ws.colexp_off),
+                     reinterpret_cast<const unsigned *>(w + c.ws.status_off) + kUnscaledWord};
   PlanPtrs p = c.ptrs();
   p.trsm_tasks += base;
-#define TS(S)                                                                       \
-  if (cols >= 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);       \
-  else launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st)
+#define TS(S)                                                                                                   \
+  if (cols >= 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);                                         \
+  else launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st);                                                   \
+  trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y)
   SC_SPLIT_SWITCH(S_, TS)
 #undef TS
   return (int)cudaGetLastError();
-}
-
-int launch_colexp_reset(const sc_ctx &c, void *ws, void *stream) {
-  int64_t ncols = 0;
-  for (int32_t m : c.m) ncols += m;
-  if (ncols <= 0) return 0;
-  uint8_t *w = static_cast<uint8_t *>(ws);
-  return (int)cudaMemsetAsync(w + c.ws.colexp_off, 0, sizeof(int) * (size_t)ncols, static_cast<cudaStream_t>(stream));
 }
 
 int launch_yslice_group(const sc_ctx &c, int S_, int64_t base, int64_t count, const double *Y, void *ws,

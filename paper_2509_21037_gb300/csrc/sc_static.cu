@@ -62,10 +62,10 @@ extern "C" sc_status sc_assemble_batch_static(sc_ctx *ctx, const double *L_value
   double *invd = reinterpret_cast<double *>(ws + ctx->ws.invd_off);
   double *Y = reinterpret_cast<double *>(ws + ctx->ws.y_off);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the array keeps the previous call's contents: only the status word must
+  // the array keeps the previous call's contents: only the status area must
   // start at zero (every Y entry a call reads is zeroed or written by its own
   // trsm tasks first, and every reciprocal diagonal by its prep kernel)
-  e = cudaMemsetAsync(status, 0, sizeof(uint32_t), st);
+  e = cudaMemsetAsync(status, 0, kStatusBytes, st);
   if (e != cudaSuccess) return static_fail(ctx, e, "sc_assemble_batch_static: status reset");
   int rc = launch_prep(*ctx, L_values_dev, invd, status, F_dev, ws, stream);
   if (rc) return static_fail(ctx, (cudaError_t)rc, "prep kernel launch");

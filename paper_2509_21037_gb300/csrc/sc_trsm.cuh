@@ -31,6 +31,10 @@ __device__ __forceinline__ void cp_async8(double *dst, const double *src, bool i
 // block): one square 180 -> 32 us, 36 plane squares 1.01 -> 0.28 ms, eight
 // elasticity cubes 20.0 -> 7.8 ms, 64 heat cubes 17.5 -> 17.4 ms (1.14 TFLOP/s of useful work).
 
+// Split precision: blocks of at most kDirect columns update the rows below in FP64, a multiply-add per
+// column and entry of Y against the two operations that an entry costs after the digit products.
+constexpr int kDirect = 4;
+
 constexpr int kTrsmCtas = 4;   // resident CTAs per SM: 128 registers a thread (at 96 and 80 they spill: 7.8 -> 8.8 ms on eight elasticity cubes)
 
 // What a warp keeps of a listed supernode.
@@ -52,8 +56,11 @@ __device__ __forceinline__ int tri_at(int row, int p) { return p * 31 - p * (p -
 // The triangle of one block with V >= wk lanes across the live columns: lane
 // = (row slot, column), NP pieces of 32 / V rows (NP a constant: a row update that
 // is only predicated off would hold the FP64 pipe all the same).  kScaled: T holds L(row, p) / L(p, p), so that
-// the chain is one multiply-add a step and the rows are divided at the end (a rounding in another place, so
-// only where the digits' error is larger than either).
+// the chain is one multiply-add a step and the rows are divided at the end.  Every entry of L is rounded once more, so
+// only the split-precision form does it, where that is lost in the digits' error (7 digits against 64 bits, six
+// subdomains of cubes, squares and elasticity: 1.6e-15 to 6.8e-15 with it and without it; on the mean 0.98 and 0.97 of
+// the error before), and only where FP64 holds the ratios in full (prep_kernel).  Without it, TRSM at 7 and 5 digits:
+// 64 heat cubes 6.4 -> 6.6 and 5.0 -> 5.4 ms, four elasticity cubes 1.43 -> 1.47 and 1.18 -> 1.34.
 template <int V, int NP, bool kScaled, class Sm>
 __device__ __forceinline__ void trsm_pieces(Sm &sm, const double *__restrict__ T, double *__restrict__ Yb, int ws, int kw, int wk,
                                             double idv, int lane) {
