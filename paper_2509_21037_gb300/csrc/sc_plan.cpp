@@ -247,7 +247,7 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
   std::vector<int32_t> active_cols;
   std::vector<int32_t> cuts;
   std::vector<int32_t> sblk_v[kNumVariants], sblk_w[kNumVariants];
-  std::vector<double> trsm_cost, syrk_cost;
+  std::vector<double> trsm_cost, syrk_cost, trsm_width, trsm_below;   // the last two: columns of a task's blocks, and each times the rows below
   std::vector<int8_t> trsm_var, syrk_var;
   std::vector<int32_t> trsm_wave, syrk_wave;
 
@@ -405,7 +405,7 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       t.list_len = (int32_t)clist[q].size();
       t.seed_lo = sub_seed_ptr[t.c_lo];
       t.seed_hi = sub_seed_ptr[t.c_lo + t.w];
-      double cost = 0, exec = 0;
+      double cost = 0, exec = 0, width = 0, below = 0;
       for (int32_t s : clist[q]) {
         trsm_list.push_back(gidx[s]);
         const SnDev &sn = sns[gidx[s]];
@@ -418,12 +418,16 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
           const double blk = kw * kw + 2.0 * kw * (nrow - kb - kw);
           cost += wkb * blk;
           exec += kChunk * blk;
+          width += kw;
+          below += kw * (nrow - kb - kw);
         }
       }
       st.flops_trsm += cost;
       st.flops_trsm_exec += exec;
       trsm.push_back(t);
       trsm_cost.push_back(exec + 1e3 * t.list_len);
+      trsm_width.push_back(width);
+      trsm_below.push_back(below);
       trsm_var.push_back(ctx->sub_var[i]);
       trsm_wave.push_back(ctx->sub_wave[i]);
     }
@@ -577,12 +581,28 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
     // columns: 64 heat cubes 22.9 / 19.8 / 18.4 / 17.9 / 17.4 (rule: 16), 8 elasticity cubes
     // 7.80 / 7.78 / 10.7 / 15.3 / 33.7 (2), 36 plane squares 0.355 / 0.280 / 0.299 / 0.425 / 0.82 (2),
     // one square 0.031 / 0.035 / 0.050 / 0.065 / 0.10 (1).
-    // The split-precision TRSM takes 2 or 4 columns per warp by the same rule (7 digits, ms at 2 / 4: 64 heat cubes
-    // 7.7 / 6.3 (rule: 4), 27 small ones 0.37 / 0.30 (4), 8 elasticity cubes 2.3 / 2.9 (2), 36 squares 0.32 / 0.39 (2)).
+    // The split-precision TRSM takes 2 or 4 columns per warp by the same rule (7 digits, ms at 2 / 4: 27 heat cubes of 11^3
+    // nodes 0.44 / 0.41 (rule: 4), 8 elasticity cubes 2.3 / 3.1 (2), 36 squares 0.35 / 0.42 (2)), or the whole chunk on one CTA
+    // (8): that form reads L's digits a half or a quarter as often, but has a barrier for every eight rows of a
+    // triangle, which the rows below the block have to pay for, and the longest tail.  With r = the longest task / a
+    // CTA slot's share (four to an SM) and b = the mean number of rows below a block's column it is taken where
+    // 300 r <= b, and for 3 and 4 digits, whose products are few, only where r <= 1.  7 digits, ms at 2 / 4 / 8 (r, b):
+    // 64 heat cubes 8.1 / 5.9 / 5.4 (0.39, 195), 27 of them 3.0 / 2.3 / 2.5 (1.03, 194), 64 elasticity cubes 30 / 22.5 / 19.2
+    // (0.61, 435), 32 of them 9.7 / 7.4 / 6.8 (1.25, 393), 16 of them 4.8 / 4.0 / 5.1 (2.5, 407), 120 small squares and 8 large
+    // cubes 20 / 16.0 / 13.9 (1.48, 794) and 13.0 / 10.4 / 11.1 (2.43, 686), 400 squares 3.8 / 3.2 / 3.7 (0.60, 41).
+    std::vector<double> width(ctx->waves.size() * kNumVariants), below(width);
+    for (int32_t k : o) {
+      width[trsm_wave[k] * kNumVariants + trsm_var[k]] += trsm_width[k];
+      below[trsm_wave[k] * kNumVariants + trsm_var[k]] += trsm_below[k];
+    }
     each_group(trsm_cost, trsm_var, trsm_wave, o, [&](sc_ctx::WaveGroups &g, int v, double total, double longest) {
       int &cols = g.trsm_cols[v];
       cols = v == 0 ? 16 : 4;
       while (cols > (v == 0 ? 1 : 2) && longest * cols / kChunk > 0.5 * total / (4 * kGridSMs)) cols /= 2;
+      if (v == 0) return;
+      const size_t k = (&g - ctx->waves.data()) * kNumVariants + v;
+      const double r = longest * (4 * kGridSMs) / total;
+      if (300.0 * r * width[k] <= below[k] && (var_digits(v) >= 5 || r <= 1.0)) cols = 8;
     });
     std::vector<TrsmTask> t2(trsm.size());
     for (size_t k = 0; k < o.size(); ++k) t2[k] = trsm[o[k]];

@@ -363,7 +363,11 @@ struct TrsmSplit {
   const unsigned *unscaled;    // not 0: triangles are not divided by their diagonal (prep_kernel)
 };
 
-// A lane's fragments of the S digit planes of L, panel rows row (va) and row + 8 (vb), by 16-byte loads (kVector) or by words.
+// A lane's fragments of the S digit planes of L, panel rows row (va) and row + 8 (vb): by words, which arrive where the
+// products need them, or (kVector) by 16-byte loads, a quarter of the loads, but their registers have to be regrouped for
+// every product.  By words / by vectors, TRSM with packing at 7 digits: 64 heat cubes 5.9 / 6.3 ms with 4 columns to a warp,
+// 5.3 / 6.2 with the whole chunk on a CTA; at 5 digits and below, and with 2 columns to a warp (8 elasticity cubes
+// 2.41 / 2.33), where the registers suffice for both, the vectors are as fast or faster.
 template <int S, bool kVector>
 struct Fragments;
 template <int S>
@@ -506,7 +510,7 @@ __device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, 
             for (int r0 = 16 * warp; r0 < nb; r0 += 16 * (kThreads / 32)) {
               const int ra = r0 + g, rb = r0 + g + 8;
               const bool va = ra < nb, vb = rb < nb;
-              Fragments<S, true> fr;
+              Fragments<S, (C < 4 || S <= 5)> fr;
               fr.load(sp, base + ra, va, vb, tg);
               const int ea = va ? sp.lexp[base + ra] : 0, eb = vb ? sp.lexp[base + rb] : 0;
               double *ta = nullptr, *tb = nullptr;                 // this lane's two target rows
@@ -600,19 +604,22 @@ __global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(co
                   *reinterpret_cast<TeamShared<C, S> *>(team_smem), threadIdx.x >> 5, threadIdx.x & 31);
 }
 
-// The same for a whole chunk of 32 columns by one CTA, the triangle shared by its warps 8 rows at a time.  Same operations in
-// the same order as trsm_team, so the same bits.  It runs behind trsm_split_kernel and takes the launch over
-// only where the triangles must not be divided by their diagonals: an empty launch otherwise.
+// The same for a whole chunk of 32 columns by one CTA, the triangle shared by its warps 8 rows at a time: the rows
+// below read L's digits once for 32 columns instead of once for 8 or 16, the first of them while one warp solves, and
+// every step of the triangle has a barrier.  Same operations in the same order as trsm_team, so the same bits.
+// always: the planner's choice for a batch of large subdomains (rule and figures in sc_plan.cpp).  Else it runs
+// behind trsm_split_kernel and takes the launch over only where the triangles must not be divided by their
+// diagonals: an empty launch otherwise.
 template <int S>
 __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_chunk_kernel(const PlanPtrs P, const double *__restrict__ Lv,
                                                                  const double *__restrict__ invd, const TrsmSplit sp,
-                                                                 double *__restrict__ Y) {
+                                                                 double *__restrict__ Y, bool always) {
   __shared__ double X[32][33];                              // the solved block: [row][live column]
   __shared__ double T[32 * 31 / 2];
   __shared__ __align__(16) __nv_bfloat16 PX[S][32][kPad];   // its digit planes: [digit][live column][row]
   __shared__ int emax[32];
   const bool unscaled = *sp.unscaled != 0;
-  if (!unscaled) return;
+  if (!always && !unscaled) return;
   const TrsmTask t = P.trsm_tasks[blockIdx.x];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, tg = lane & 3;
@@ -836,9 +843,9 @@ int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t c
   PlanPtrs p = c.ptrs();
   p.trsm_tasks += base;
 #define TS(S)                                                                                                   \
-  if (cols >= 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);                                         \
-  else launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st);                                                   \
-  trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y)
+  if (cols == 2) launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st);                                         \
+  else if (cols == 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);                                    \
+  trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y, cols >= 8)
   SC_SPLIT_SWITCH(S_, TS)
 #undef TS
   return (int)cudaGetLastError();
