@@ -70,8 +70,12 @@ constexpr int kApplyWarps = 4;                     // warps per CTA
 
 // In FP64 two stages per warp and 12 warps per SM: a warp's next tile arrives while its multiply-adds hold the
 // FP64 pipe (64 heat cubes 197 us, with one stage and 20 warps 203).  In fixed point one stage and 24 warps, whose
-// integer chains need the others (64 heat cubes 146 us and a quarter in FP64 128; 20 warps 150 and 133; two stages and
-// 12 warps 174 and 158); the limbs of lambda block J lie over the block itself so that six CTAs fit an SM.
+// integer chains need the others (64 heat cubes, before the 16-byte accesses below: 146 us and a quarter in FP64 128; 20
+// warps 150 and 133; two stages and 12 warps 174 and 158); the limbs of lambda block J lie over the block itself so that six CTAs fit an SM.
+// From 64 tiles per resident warp on, the fixed-point runs are handed out in rounds of 32 to 63 tiles: SMs take different
+// times for as many tiles, and with one run to a warp all wait for the slowest (512 elasticity cubes 3127 -> 2830 us, 2048
+// mixed subdomains 11.25 -> 10.05 ms; 2048 in runs of 128 10.09, of 512 10.77).  FP64 runs gain nothing (4708 us and, in
+// runs of 32, 4735 on the 512 cubes).
 template <bool kFixed>
 struct ApplyShape {
   static constexpr int kStages = kFixed ? 1 : 2, kCtas = kFixed ? 6 : 3;
@@ -95,9 +99,9 @@ struct ApplyWarp {
 // kFixed: of every four tiles of a row block fp64_quarters (0..4) are multiplied in FP64 (FP64 pipe) and the
 // rest in fixed point (integer pipes), so that both pipes work at once; else all in FP64.
 // Bound by the FP64 pipe (64 multiply-adds of 16 cycles a tile and SM: 173 us for 64 heat cubes), in fixed point by
-// integer issue.  64 heat cubes (437 MB): FP64 246 -> 197 us, fixed 177 -> 144, a quarter in FP64 168 -> 127 (3.4 TB/s);
-// 710 tiles: 31 -> 15 us; 657,000 tiles, where the ends of the runs don't count: FP64 2383 -> 2295, fixed 1576 both,
-// a quarter in FP64 1480 -> 1347.
+// integer issue.  Against a CTA per (subdomain, row block), 64 heat cubes (437 MB): FP64 243 -> 199 us, fixed 176 -> 140, a
+// quarter in FP64 167 -> 124 (3.5 TB/s); 710 tiles: FP64 31 -> 15 us; 657,000 tiles: FP64 2380 -> 2298, fixed 1569 -> 1407, a
+// quarter 1472 -> 1271; 2048 mixed subdomains: 17.3 -> 16.95 ms, 11.2 -> 10.05, 10.5 -> 9.0.
 template <bool kFixed>
 __global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
     apply_tiles_kernel(const PlanPtrs P, int64_t n_tasks, int64_t n_tiles, const double *__restrict__ F,
@@ -183,15 +187,25 @@ __global__ void __launch_bounds__(32 * kApplyWarps, ApplyShape<kFixed>::kCtas)
         if (qJ >= 0) atomicAdd(q + qJ, z0 + z1);
       }
     } else if constexpr (kFixed) {
+      // The cut to fixed point goes entry by entry, so a lane takes the pairs of rows that a 16-byte access holds:
+      // half the shared-memory instructions of one entry at a time (512 elasticity cubes, one run to a warp, 3220 -> 3131 us).
+      const int e0 = (lane >> 4) * kStride + 2 * (lane & 15);
       uint32_t em = 0;                             // the largest high word holds the largest exponent
 #pragma unroll 8
-      for (int c = 0; c < 32; ++c) em = max(em, (uint32_t)__double2hiint(T[c * kStride + lane]) & 0x7FFFFFFFu);
+      for (int c = 0; c < 32; c += 2) {
+        const double2 v = *reinterpret_cast<const double2 *>(&T[c * kStride + e0]);
+        em = max(em, max((uint32_t)__double2hiint(v.x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v.y) & 0x7FFFFFFFu));
+      }
       const uint32_t exT = __reduce_max_sync(kFull, em) >> 20;
       const uint32_t exJ = __reduce_max_sync(kFull, exp_field(p));
       if (exT != 0) {                              // an all-zero tile adds nothing (uniform)
-        int2 *Tl = reinterpret_cast<int2 *>(T);    // each lane converts its row, in place
+        int2 *Tl = reinterpret_cast<int2 *>(T);    // the limbs in place of the entries
 #pragma unroll 8
-        for (int c = 0; c < 32; ++c) Tl[c * kStride + lane] = fixed_limbs(T[c * kStride + lane], exT);
+        for (int c = 0; c < 32; c += 2) {
+          const double2 v = *reinterpret_cast<const double2 *>(&T[c * kStride + e0]);
+          const int2 x = fixed_limbs(v.x, exT), y1 = fixed_limbs(v.y, exT);
+          *reinterpret_cast<int4 *>(&Tl[c * kStride + e0]) = make_int4(x.x, x.y, y1.x, y1.y);
+        }
         sm.lJ[lane] = fixed_limbs(p, exJ);
         __syncwarp();
         if (exJ != 0) {
@@ -241,7 +255,9 @@ cudaError_t launch_tiles(const sc_ctx &c, const double *F, const double *lam, do
   constexpr int smem = (int)sizeof(ApplyWarp<ApplyShape<kFixed>::kStages>) * kApplyWarps;
   cudaError_t e = cudaFuncSetAttribute(apply_tiles_kernel<kFixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int64_t grid = std::min<int64_t>((int64_t)kGridSMs * ApplyShape<kFixed>::kCtas, (nt + kApplyWarps - 1) / kApplyWarps);
+  int64_t grid = std::min<int64_t>((int64_t)kGridSMs * ApplyShape<kFixed>::kCtas, (nt + kApplyWarps - 1) / kApplyWarps);
+  // fixed point: several rounds of runs of 32 to 63 tiles (see ApplyShape)
+  if (kFixed) grid *= std::max<int64_t>(1, nt / (kApplyWarps * grid * 32));
   apply_tiles_kernel<kFixed><<<(unsigned)grid, 32 * kApplyWarps, smem, st>>>(c.ptrs(), c.n_apply, nt, F, lam, q,
                                                                            fp64_quarters);
   return cudaGetLastError();
