@@ -15,7 +15,7 @@ def _factors(name):
         assert fs[0].m == 0
         return [fs[0], fs[3], fs[0], fs[0], fs[1], fs[0]]
     if name == "squares":
-        return host.factorize_problem(synth.mixed_batch((2, 1), (12, 17), (1, 1, 1), (2, 2), 3).subdomains)
+        return host.factorize_problem(synth.mixed_batch((2, 2), (20, 33), (1, 1, 1), (2, 2), 3).subdomains)
     return host.factorize_problem(synth.cube_heat_3d(parts=2, k=6).subdomains[:2])   # supernodes of up to 49 columns
 
 
