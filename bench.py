@@ -164,7 +164,7 @@ class ClockSampler:
 
 
 # the source files of each profiled kernel
-_KERNEL_SOURCE = {"syrk_kernel": ("sc_kernels.cu",), "trsm_kernel": ("sc_kernels.cu", "sc_trsm.cuh"),
+_KERNEL_SOURCE = {"syrk_kernel": ("sc_kernels.cu", "sc_trsm.cuh"), "trsm_kernel": ("sc_kernels.cu", "sc_trsm.cuh"),
                   "apply_tiles_kernel": ("sc_apply_fixed.cu", "sc_tiles.cuh"),
                   "apply_digits_kernel": ("sc_apply_digits.cu", "sc_tiles.cuh"),
                   "tier_kernel": ("sc_implicit.cu",)}

@@ -113,7 +113,7 @@ sc_status sci_apply(sci_ctx *ctx, const double *L_values_dev, const double *lamb
 sc_status sci_device_status(sci_ctx *ctx, const void *ws_dev, void *stream);
 
 /* Host copy of the plan tables (bytes >= plan_bytes), for inspection.  Layout:
- * a 256-byte header {uint32 magic 'SCIP', uint32 version 1, int32 nsub, pad,
+ * a 256-byte header {uint32 magic 'SCIP', uint32 version 2, int32 nsub, pad,
  * int64 n_sn, n_levptr, n_rows, n_grow, n_gent, n_sent, n_items,
  * uint64 sec_off[8], piece_off, int64 n_pieces} and nine 256-byte aligned
  * sections: subdomains (64 B each, largest first: int64 x_off; int32 n, sn_lo,
@@ -122,7 +122,8 @@ sc_status sci_device_status(sci_ctx *ctx, const void *ws_dev, void *stream);
  * level boundaries (int32), pruned rows (int32), gather rows (int32 r, e_lo,
  * e_hi, pad), gather entries (int32 gj, sign), scatter entries (int32 r, gj,
  * sign, pad), cluster items (int32 kind, n, sub[8]; kind 0: sub[0] on the
- * whole cluster, kind 1: sub[r] on CTA r for r < n),
+ * whole cluster, kind 1: sub[r] on CTA r for r < n, kind 2: sub[j] on the CTA
+ * pair (2j, 2j + 1) for j < n),
  * pieces of the tiered schedule (int32 sub, lev_lo, n_lev, s_lo, s_hi, pad; tier
  * by tier: levels and scatter entries as in the subdomains). */
 sc_status sci_export_plan(const sci_ctx *ctx, void *dst, size_t bytes);

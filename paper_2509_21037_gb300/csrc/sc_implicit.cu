@@ -9,7 +9,7 @@
 // gather and by entry for the scatter.
 //
 // Device side: a tiered schedule by default (see "the tiered schedule" below:
-// 64 heat cubes 1.45 -> 0.75 ms); clusters or CTA pairs where the options ask
+// 64 heat cubes 1.43 -> 0.79 ms); clusters or CTA pairs where the options ask
 // for them, then one launch with one CTA per subdomain otherwise.
 // Forward solve level by level upwards, backward solve level by level downwards, the warps sharing
 // the supernodes of a level; a barrier between levels.  A warp solves its
@@ -886,9 +886,9 @@ __global__ void __launch_bounds__(kThreadsI, 1) implicit_kernel(const IPtrs P, c
 // subdomains than SMs and works through the tree's wide lower part on one
 // SM.  Here every subdomain's visited tree is cut into tiers of pieces (the
 // planner, tier_pieces): small subtrees, then the middle of the tree, then the top
-// separators.  One launch per tier and direction, one CTA per piece: forward
-// tier 0, 1, .., the top forward and backward in one, then backward down
-// the tiers.  Pieces of a tier share no rows; their updates of rows above are
+// separators.  One launch per tier that has pieces and direction, one CTA per piece: forward
+// tier 0, 1, .., then backward down the tiers; the last tier, where it has pieces, runs forward and backward
+// in one (on 64 heat cubes it has none: the caps leave nothing above the third, six launches).  Pieces of a tier share no rows; their updates of rows above are
 // atomic and read by later launches only, so no CTA waits for another.
 
 // q = 0, x = B^T lambda (x is zero on entry) and the reciprocal diagonals of the visited columns.
@@ -1390,9 +1390,14 @@ sc_status build(sci_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d, int64_t 
   const bool want_pairs = pairs == 1;
   // The tiers' caps: halves of the largest subdomain's entries (a nested-dissection tree halves its
   // subtrees level by level), not below a quarter of an SM's share of the batch nor 4000 entries, which a
-  // CTA works through in about the time of a launch.  GB300, us with 1 / 2 / 3 / 4 / 5 tiers: 64 heat cubes
-  // 1130 / 758 / 772 / 807 / 900, 8 elasticity cubes and 16 squares 2055 / 1502 / 1564 / 1314 / 1563, four elasticity
-  // cubes 1640 / 1620 / 1407 / 1414 / 1111, 36 squares 430 / 475 / 294 / 314 / 322.
+  // CTA works through in about the time of a launch.  GB300, us with 1 / 2 / 3 / 4 / 5 tiers (an earlier form of the
+  // kernels): 64 heat cubes 1130 / 758 / 772 / 807 / 900, 8 elasticity cubes and 16 squares 2055 / 1502 / 1564 / 1314 /
+  // 1563, four elasticity cubes 1640 / 1620 / 1407 / 1414 / 1111, 36 squares 430 / 475 / 294 / 314 / 322.  No count is best for
+  // all; the rule takes as many as the sizes allow, at most four, up to 7 % behind the best of two to four, and four
+  // elasticity cubes would gain by a fifth.
+  // Against clusters of 8 CTAs for the subdomains above twice the even share, ms: 120 squares with 8 large elasticity cubes
+  // 7.06 -> 5.8, 264 mixed 5.93 -> 4.4, 2 cubes of 21^3 nodes among 64 squares 4.29 -> 3.05; against one launch with a CTA to
+  // a subdomain: 512 elasticity cubes 14.7 -> 9.3, 2048 mixed 38.5 -> 33.9.
   int64_t cap[kTiers - 1] = {};
   if (ctx->tiered && nsub > 0) {
     const double least = std::max((double)nnz_all / (4 * kCtaSlots), 4000.0);

@@ -68,7 +68,7 @@ struct SnDev {
 struct TrsmTask {
   int32_t sub, c_lo, w;       // sorted columns [c_lo, c_lo + w)
   int32_t list_off, list_len; // supernodes touched, ascending (children first)
-  int32_t seed_lo, seed_hi;   // seeds of these columns
+  int32_t seed_lo, seed_hi;   // seeds of these columns (parts of a task find theirs through seed_ptr)
   int32_t pad;
 };
 

@@ -5,7 +5,9 @@
 //                    NOT_SPD bit of the workspace status word (paper Sec. 3.1:
 //                    the factor is copied in; here its CSC columns are read
 //                    in place, because a fundamental supernode's CSC column is
-//                    already a dense trapezoidal panel column).
+//                    already a dense trapezoidal panel column); F's padding,
+//                    and for split precision Y's column bounds and a look at
+//                    the triangles' range.
 //   trsm_kernel   -- Y = L^{-1} P B^T on a part of a 32-column chunk of the
 //                    pivot-sorted columns (paper Sec. 3.2), one warp to a part:
 //                    zero + seed the part's nonzero rows of Y, then for each

@@ -349,11 +349,10 @@ __global__ void __launch_bounds__(kThreads, (S <= 5 ? 4 : 3)) syrk_split_kernel(
 // is the CTA's: its columns' digit planes in shared memory, the rows' m-tiles dealt to the
 // warps, each L fragment used for all of the CTA's columns.  Narrow CTAs (C = 2) have
 // the shorter triangles and fill the GPU on small batches; C is chosen as the FP64 TRSM's
-// columns per warp are (sc_plan.cpp).  Bound by the FP64 pipe (triangles, and two
+// columns per warp are (sc_plan.cpp).  Batches of large subdomains take trsm_chunk_kernel below.  Bound by the FP64 pipe (triangles, and two
 // operations per entry and block after the digit products) and by latency.  Against one CTA
 // per 32-column chunk whose warps shared each triangle 8 columns at a time, 7 digits, TRSM with its packing:
-// one square 312 -> 64 us, 36 squares 1.11 -> 0.33 ms, 8 elasticity cubes 4.04 -> 2.31 ms,
-// 64 heat cubes 6.05 -> 6.35 ms (their SYRK stage gains 0.14 ms: the columns' bounds come from here).
+// one square 312 -> 64 us, 36 squares 1.11 -> 0.33 ms, 8 elasticity cubes 4.04 -> 2.31 ms.
 
 struct TrsmSplit {
   const __nv_bfloat16 *Ld;     // digit planes of L
@@ -591,8 +590,9 @@ __device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, 
   }
 }
 
-// Resident CTAs: with C = 2 three (168 registers, no spills: 2.9 -> 2.3 ms on eight elasticity cubes at 7 digits),
-// with C = 4 four (6.6 -> 6.3 ms on 64 heat cubes).
+// Resident CTAs: with C = 2 three (168 registers, 8 bytes of spills at 7 digits and none below: 2.9 -> 2.3 ms on eight
+// elasticity cubes at 7 digits), with C = 4 four (128 registers, 128 / 72 / 32 bytes of spills at 7 / 6 / 5 digits and still
+// 6.6 -> 6.3 ms on 64 heat cubes at 7).
 template <int C, int S>
 __global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(const PlanPtrs P, const double *__restrict__ Lv,
                                                               const double *__restrict__ invd, const TrsmSplit sp,

@@ -35,7 +35,9 @@ __device__ __forceinline__ void cp_async8(double *dst, const double *src, bool i
 // column and entry of Y against the two operations that an entry costs after the digit products.
 constexpr int kDirect = 4;
 
-constexpr int kTrsmCtas = 4;   // resident CTAs per SM: 128 registers a thread (at 96 and 80 they spill: 7.8 -> 8.8 ms on eight elasticity cubes)
+// Resident CTAs per SM: 128 registers a thread, with which W = 16 spills 84 bytes and the others none; at 96 and 80 all do
+// (7.8 -> 8.8 ms on eight elasticity cubes).
+constexpr int kTrsmCtas = 4;
 
 // What a warp keeps of a listed supernode.
 struct TrsmSn {
