@@ -152,7 +152,7 @@ sc_status sc_assemble_batch(sc_ctx *ctx, const double *L_values_dev, double *F_d
   double *invd = reinterpret_cast<double *>(ws + ctx->ws.invd_off);
   double *Y = reinterpret_cast<double *>(ws + ctx->ws.y_off);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemsetAsync(status, 0, kStatusBytes, st);
+  cudaError_t e = cudaMemsetAsync(status, 0, ctx->n_slices > 0 ? kStatusBytes : sizeof(uint32_t), st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "sc_assemble_batch status reset");
   record(ctx, 0, st);
   int rc = launch_prep(*ctx, L_values_dev, invd, status, F_dev, ws, stream);

@@ -45,6 +45,7 @@ namespace sc {
 // look at the triangles, a warp to a (supernode, block).  Where an entry is so far from its column's diagonal (rows of L
 // that differ by hundreds of orders of magnitude) that FP64 may not hold their ratio in full, the
 // split TRSM must not divide its triangles by the diagonal.
+template <bool kSplit>
 __global__ void __launch_bounds__(256) prep_kernel(const int64_t *__restrict__ lcp, const int32_t *__restrict__ active,
                                                    int64_t nact, int nprep, const double *__restrict__ Lv,
                                                    double *__restrict__ invd, uint32_t *__restrict__ status,
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const int64_t *__restrict__ l
     }
     return;
   }
-  if ((int)blockIdx.x >= nprep + nsub) {
+  if (kSplit && (int)blockIdx.x >= nprep + nsub) {
     const int64_t cta = blockIdx.x - nprep - nsub, nt = (int64_t)(gridDim.x - nprep - nsub) * blockDim.x;
     for (int64_t k = cta * blockDim.x + threadIdx.x; k < ncols; k += nt) colexp[k] = 0;
     const int64_t item = cta * (blockDim.x / 32) + threadIdx.x / 32;
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const int64_t *__restrict__ l
     // high words; entry (t, q) of the triangle at q nr - q (q + 1) / 2 + t
     const uint32_t *Lh = reinterpret_cast<const uint32_t *>(Lv + lcp[s.lcp_off + kb]) + 1;
     bool out = false;
-#pragma unroll 8
+#pragma unroll 16
     for (int q = 0; q < kw; ++q) {
       const int o = q * nr - q * (q + 1) / 2;
       const uint32_t l = r > q && r < kw ? Lh[2 * (o + r)] : 0u, d = r > q && r < kw ? Lh[2 * (o + q)] : 0u;
@@ -394,10 +395,12 @@ int launch_prep(const sc_ctx &c, const double *Lv, double *invd, uint32_t *statu
     for (int32_t m : c.m) ncols += m;
     ncheck = std::max<int64_t>((c.n_sblk + 7) / 8, ncols > 0);
   }
-  if (nprep + c.nsub > 0)
-    prep_kernel<<<(unsigned)(nprep + c.nsub + ncheck), 256, 0, S(stream)>>>(
+  if (nprep + c.nsub > 0) {
+    auto kernel = c.n_slices > 0 ? prep_kernel<true> : prep_kernel<false>;
+    kernel<<<(unsigned)(nprep + c.nsub + ncheck), 256, 0, S(stream)>>>(
         p.lcp, p.active_cols, c.n_active_cols, nprep, Lv, invd, status, p.subs, c.nsub, F, p, c.n_sblk,
         reinterpret_cast<int *>(static_cast<uint8_t *>(ws) + c.ws.colexp_off), ncols);
+  }
   return (int)cudaGetLastError();
 }
 

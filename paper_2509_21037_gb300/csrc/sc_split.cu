@@ -34,6 +34,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "sc_digits.cuh"
@@ -590,42 +591,30 @@ __device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, 
   }
 }
 
-// Resident CTAs: with C = 2 three (168 registers, 8 bytes of spills at 7 digits and none below: 2.9 -> 2.3 ms on eight
-// elasticity cubes at 7 digits), with C = 4 four (128 registers, 128 / 72 / 32 bytes of spills at 7 / 6 / 5 digits and still
-// 6.6 -> 6.3 ms on 64 heat cubes at 7).
-template <int C, int S>
-__global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(const PlanPtrs P, const double *__restrict__ Lv,
-                                                              const double *__restrict__ invd, const TrsmSplit sp,
-                                                              double *__restrict__ Y) {
-  extern __shared__ __align__(16) unsigned char team_smem[];
-  constexpr int kParts = kChunk / (4 * C);
-  if (*sp.unscaled) return;                                        // trsm_chunk_kernel takes the whole launch
-  trsm_team<C, S>(P, P.trsm_tasks[blockIdx.x / kParts], blockIdx.x % kParts, Lv, invd, sp, Y,
-                  *reinterpret_cast<TeamShared<C, S> *>(team_smem), threadIdx.x >> 5, threadIdx.x & 31);
-}
-
 // The same for a whole chunk of 32 columns by one CTA, the triangle shared by its warps 8 rows at a time: the rows
 // below read L's digits once for 32 columns instead of once for 8 or 16, the first of them while one warp solves, and
 // every step of the triangle has a barrier.  Same operations in the same order as trsm_team, so the same bits.
-// always: the planner's choice for a batch of large subdomains (rule and figures in sc_plan.cpp).  Else it runs
-// behind trsm_split_kernel and takes the launch over only where the triangles must not be divided by their
-// diagonals: an empty launch otherwise.
+// The planner takes it for batches of large subdomains (trsm_chunk_kernel; rule and figures in sc_plan.cpp).  Where the
+// triangles must not be divided by their diagonals it stands in for trsm_team: a CTA per task behind the team's in the
+// same launch, which otherwise returns at once.  A launch of its own cost 3 to 5 us of a small assembly's 75 to 110, and
+// inlined into trsm_split_kernel it took up to 3 % of the teams' speed at 5 and 6 digits.
 template <int S>
-__global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_chunk_kernel(const PlanPtrs P, const double *__restrict__ Lv,
-                                                                 const double *__restrict__ invd, const TrsmSplit sp,
-                                                                 double *__restrict__ Y, bool always) {
-  __shared__ double X[32][33];                              // the solved block: [row][live column]
-  __shared__ double T[32 * 31 / 2];
-  __shared__ __align__(16) __nv_bfloat16 PX[S][32][kPad];   // its digit planes: [digit][live column][row]
-  __shared__ int emax[32];
-  const bool unscaled = *sp.unscaled != 0;
-  if (!always && !unscaled) return;
-  const TrsmTask t = P.trsm_tasks[blockIdx.x];
+struct ChunkShared {
+  double X[32][33];                              // the solved block: [row][live column]
+  double T[32 * 31 / 2];
+  __align__(16) __nv_bfloat16 PX[S][32][kPad];   // its digit planes: [digit][live column][row]
+  int emax[32];
+};
+
+template <int S>
+__device__ __noinline__ void trsm_chunk(const PlanPtrs &P, int task, const double *__restrict__ Lv, const double *__restrict__ invd,
+                           const TrsmSplit &sp, double *__restrict__ Y, ChunkShared<S> &sm, bool unscaled) {
+  const TrsmTask t = P.trsm_tasks[task];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, tg = lane & 3;
   const int c_hi = t.c_lo + t.w;
   // the warp that solves: spread over the SM's sub-partitions across co-resident CTAs
-  const int tri = (int)((blockIdx.x * 2654435761u) >> 30);
+  const int tri = (int)(((unsigned)task * 2654435761u) >> 30);
   int *colexp = sp.colexp + P.subs[t.sub].col_off;
   for (int li = 0; li < t.list_len; ++li) {
     const SnDev s = P.sns[P.trsm_list[t.list_off + li]];
@@ -659,14 +648,14 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
       if (pre) load_fr(16 * warp);
       for (int e = tid; e < kw * 32; e += kThreads) {
         const int q = e >> 5, c = e & 31;
-        X[q][c] = c < wk ? Ys[(int64_t)(kb + q) * ws + c] : 0.0;
+        sm.X[q][c] = c < wk ? Ys[(int64_t)(kb + q) * ws + c] : 0.0;
       }
       const bool scaled = kw > kDirect && !unscaled;
 #pragma unroll 4
       for (int p = warp; p < kw; p += kThreads / 32)
         if (lane > p && lane < kw) {
           const double l = Lc[kb + lane + p * (nr - kb - 1) - p * (p - 1) / 2];
-          T[tri_at(lane, p)] = scaled ? l * id[kb + p] : l;
+          sm.T[tri_at(lane, p)] = scaled ? l * id[kb + p] : l;
         }
       __syncthreads();
       for (int p0 = 0; p0 < kw; p0 += 8) {
@@ -674,30 +663,30 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
         if (warp == tri && lane < wk) {
           double x[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) x[i] = p0 + i < kw ? X[p0 + i][lane] : 0.0;
+          for (int i = 0; i < 8; ++i) x[i] = p0 + i < kw ? sm.X[p0 + i][lane] : 0.0;
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             if (p0 + i >= kw) break;                         // uniform
             if (!scaled) x[i] *= id[kb + p0 + i];
 #pragma unroll
             for (int r = i + 1; r < 8; ++r)
-              if (p0 + r < kw) x[r] = fma(-T[tri_at(p0 + r, p0 + i)], x[i], x[r]);
+              if (p0 + r < kw) x[r] = fma(-sm.T[tri_at(p0 + r, p0 + i)], x[i], x[r]);
           }
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            if (p0 + i < kw) X[p0 + i][lane] = x[i];
+            if (p0 + i < kw) sm.X[p0 + i][lane] = x[i];
         }
         __syncthreads();
         if (pe < kw) {                                       // then pe == p0 + 8
           if (lane < wk) {
             double x[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = X[p0 + i][lane];
+            for (int i = 0; i < 8; ++i) x[i] = sm.X[p0 + i][lane];
             for (int r = pe + ((warp - tri) & 3); r < kw; r += kThreads / 32) {
-              double xr = X[r][lane];
+              double xr = sm.X[r][lane];
 #pragma unroll
-              for (int i = 0; i < 8; ++i) xr = fma(-T[tri_at(r, p0 + i)], x[i], xr);
-              X[r][lane] = xr;
+              for (int i = 0; i < 8; ++i) xr = fma(-sm.T[tri_at(r, p0 + i)], x[i], xr);
+              sm.X[r][lane] = xr;
             }
           }
           __syncthreads();
@@ -707,12 +696,12 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
         int em = 0;
         if (lane < wk)
           for (int q = 0; q < kw; ++q) {
-            double v = X[q][lane];
-            if (scaled) X[q][lane] = v = v * id[kb + q];
+            double v = sm.X[q][lane];
+            if (scaled) sm.X[q][lane] = v = v * id[kb + q];
             Ys[(int64_t)(kb + q) * ws + lane] = v;
             em = max(em, biased_exponent(v));
           }
-        emax[lane] = em;
+        sm.emax[lane] = em;
         if (lane < wk && em) atomicMax(colexp + a + lane, em);
       }
       __syncthreads();
@@ -726,7 +715,7 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
           double acc = *tgt;
           int o = p;
           for (int q = 0; q < kw; ++q) {
-            acc = fma(-Lc[o], X[q][cl], acc);
+            acc = fma(-Lc[o], sm.X[q][cl], acc);
             o += nr - (kb + q) - 1;
           }
           *tgt = acc;
@@ -742,10 +731,10 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
       }
       for (int e = tid; e < 32 * 32; e += kThreads) {
         const int q = e >> 5, c = e & 31;
-        const double v = (q < kw && c < wk) ? X[q][c] : 0.0;
-        const uint64_t m = fixed_point(v, emax[c]);
+        const double v = (q < kw && c < wk) ? sm.X[q][c] : 0.0;
+        const uint64_t m = fixed_point(v, sm.emax[c]);
 #pragma unroll
-        for (int d = 0; d < S; ++d) PX[d][c][q] = digit_bf16(m, d, v < 0.0);
+        for (int d = 0; d < S; ++d) sm.PX[d][c][q] = digit_bf16(m, d, v < 0.0);
       }
       __syncthreads();
       for (int r0 = 16 * warp; r0 < nb; r0 += 16 * (kThreads / 32)) {
@@ -774,7 +763,7 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
             float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int q = 0; q <= d; ++q) {
-              const __nv_bfloat16 *px = &PX[d - q][8 * nt + g][2 * tg];
+              const __nv_bfloat16 *px = &sm.PX[d - q][8 * nt + g][2 * tg];
               fr.mma(c, q, px);
             }
 #pragma unroll
@@ -785,7 +774,7 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
             const int col = 8 * nt + 2 * tg + (r & 1);
             double *p = (r & 2) ? tb : ta;
             if (p && col < wk) {
-              const int e = ((r & 2 ? eb : ea) - 1022) + (emax[col] - 1022) + Groups<S>::kBlockShift;
+              const int e = ((r & 2 ? eb : ea) - 1022) + (sm.emax[col] - 1022) + Groups<S>::kBlockShift;
               const double v = (double)gr[r].block_int();
               p[col] = (e >= -1022 && e <= 1023) ? fma(-v, pow2i(e), yv[r]) : yv[r] - ldexp(v, e);
             }
@@ -795,6 +784,32 @@ __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_ch
       __syncthreads();
     }
   }
+}
+
+// Resident CTAs: with C = 2 three (168 registers, 8 bytes of spills at 7 digits and none below: 2.9 -> 2.3 ms on eight
+// elasticity cubes at 7 digits), with C = 4 four (128 registers, 128 / 72 / 32 bytes of spills at 7 / 6 / 5 digits and still
+// 6.6 -> 6.3 ms on 64 heat cubes at 7).
+template <int C, int S>
+__global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(const PlanPtrs P, const double *__restrict__ Lv,
+                                                              const double *__restrict__ invd, const TrsmSplit sp,
+                                                              double *__restrict__ Y, int n_team) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  constexpr int kParts = kChunk / (4 * C);
+  if ((int)blockIdx.x >= n_team) {                                 // a CTA per task behind them
+    if (*sp.unscaled) trsm_chunk<S>(P, (int)blockIdx.x - n_team, Lv, invd, sp, Y, *reinterpret_cast<ChunkShared<S> *>(team_smem), true);
+    return;
+  }
+  if (*sp.unscaled) return;
+  trsm_team<C, S>(P, P.trsm_tasks[blockIdx.x / kParts], blockIdx.x % kParts, Lv, invd, sp, Y,
+                  *reinterpret_cast<TeamShared<C, S> *>(team_smem), threadIdx.x >> 5, threadIdx.x & 31);
+}
+
+template <int S>
+__global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_chunk_kernel(const PlanPtrs P, const double *__restrict__ Lv,
+                                                                 const double *__restrict__ invd, const TrsmSplit sp,
+                                                                 double *__restrict__ Y) {
+  __shared__ ChunkShared<S> sm;
+  trsm_chunk<S>(P, blockIdx.x, Lv, invd, sp, Y, sm, *sp.unscaled != 0);
 }
 
 }  // namespace
@@ -826,9 +841,9 @@ int launch_lpack_split(const sc_ctx &c, int S_, int64_t base, int64_t count, con
 template <int C, int S>
 static void launch_team(const PlanPtrs &p, int n, const double *Lv, const double *invd, const TrsmSplit &sp, double *Y,
                         cudaStream_t st) {
-  const int smem = (int)sizeof(TeamShared<C, S>);
+  const int smem = (int)std::max(sizeof(TeamShared<C, S>), sizeof(ChunkShared<S>)), n_team = n * (kChunk / (4 * C));
   cudaFuncSetAttribute(trsm_split_kernel<C, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  trsm_split_kernel<C, S><<<(unsigned)(n * (kChunk / (4 * C))), kThreads, smem, st>>>(p, Lv, invd, sp, Y);
+  trsm_split_kernel<C, S><<<(unsigned)(n_team + n), kThreads, smem, st>>>(p, Lv, invd, sp, Y, n_team);
 }
 
 int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t count, const double *Lv,
@@ -845,7 +860,7 @@ int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t c
 #define TS(S)                                                                                                   \
   if (cols == 2) launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st);                                         \
   else if (cols == 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);                                    \
-  trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y, cols >= 8)
+  else trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y)
   SC_SPLIT_SWITCH(S_, TS)
 #undef TS
   return (int)cudaGetLastError();
