@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const int64_t *__restrict__ l
     // high words; entry (t, q) of the triangle at q nr - q (q + 1) / 2 + t
     const uint32_t *Lh = reinterpret_cast<const uint32_t *>(Lv + lcp[s.lcp_off + kb]) + 1;
     bool out = false;
-#pragma unroll 16
+#pragma unroll 8
     for (int q = 0; q < kw; ++q) {
       const int o = q * nr - q * (q + 1) / 2;
       const uint32_t l = r > q && r < kw ? Lh[2 * (o + r)] : 0u, d = r > q && r < kw ? Lh[2 * (o + q)] : 0u;

@@ -586,10 +586,11 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
     // (8): that form reads L's digits a half or a quarter as often, but has a barrier for every eight rows of a
     // triangle, which the rows below the block have to pay for, and the longest tail.  With r = the longest task / a
     // CTA slot's share (four to an SM) and b = the mean number of rows below a block's column it is taken where
-    // 300 r <= b, and for 3 and 4 digits, whose products are few, only where r <= 1.  7 digits, ms at 2 / 4 / 8 (r, b):
+    // b >= max(300 r, 180), and for 3 and 4 digits, whose products are few, only where r <= 1.  7 digits, ms at 2 / 4 / 8 (r, b):
     // 64 heat cubes 8.1 / 5.9 / 5.4 (0.39, 195), 27 of them 3.0 / 2.3 / 2.5 (1.03, 194), 64 elasticity cubes 30 / 22.5 / 19.2
     // (0.61, 435), 32 of them 9.7 / 7.4 / 6.8 (1.25, 393), 16 of them 4.8 / 4.0 / 5.1 (2.5, 407), 120 small squares and 8 large
-    // cubes 20 / 16.0 / 13.9 (1.48, 794) and 13.0 / 10.4 / 11.1 (2.43, 686), 400 squares 3.8 / 3.2 / 3.7 (0.60, 41).
+    // cubes 20 / 16.0 / 13.9 (1.48, 794) and 13.0 / 10.4 / 11.1 (2.43, 686), 64 elasticity cubes of 6^3 to 9^3 nodes 2.0 /
+    // 1.50 / 1.54 (1.46, 133), 400 squares 3.8 / 3.2 / 3.7 (0.60, 41).
     std::vector<double> width(ctx->waves.size() * kNumVariants), below(width);
     for (int32_t k : o) {
       width[trsm_wave[k] * kNumVariants + trsm_var[k]] += trsm_width[k];
@@ -602,7 +603,7 @@ sc_status build_plan(sc_ctx *ctx, int32_t nsub, const sc_subdomain_desc *d) {
       if (v == 0) return;
       const size_t k = (&g - ctx->waves.data()) * kNumVariants + v;
       const double r = longest * (4 * kGridSMs) / total;
-      if (300.0 * r * width[k] <= below[k] && (var_digits(v) >= 5 || r <= 1.0)) cols = 8;
+      if (std::max(300.0 * r, 180.0) * width[k] <= below[k] && (var_digits(v) >= 5 || r <= 1.0)) cols = 8;
     });
     std::vector<TrsmTask> t2(trsm.size());
     for (size_t k = 0; k < o.size(); ++k) t2[k] = trsm[o[k]];

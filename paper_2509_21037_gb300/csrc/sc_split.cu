@@ -594,10 +594,10 @@ __device__ __forceinline__ void trsm_team(const PlanPtrs &P, const TrsmTask &t, 
 // The same for a whole chunk of 32 columns by one CTA, the triangle shared by its warps 8 rows at a time: the rows
 // below read L's digits once for 32 columns instead of once for 8 or 16, the first of them while one warp solves, and
 // every step of the triangle has a barrier.  Same operations in the same order as trsm_team, so the same bits.
-// The planner takes it for batches of large subdomains (trsm_chunk_kernel; rule and figures in sc_plan.cpp).  Where the
-// triangles must not be divided by their diagonals it stands in for trsm_team: a CTA per task behind the team's in the
-// same launch, which otherwise returns at once.  A launch of its own cost 3 to 5 us of a small assembly's 75 to 110, and
-// inlined into trsm_split_kernel it took up to 3 % of the teams' speed at 5 and 6 digits.
+// The planner takes it for batches of large subdomains (rule and figures in sc_plan.cpp).  Where the triangles must not
+// be divided by their diagonals it runs behind trsm_split_kernel and takes the launch over; on ordinary factors that
+// launch is empty, 3 to 4 us of a small assembly's 75 to 110.  As part of trsm_split_kernel, inlined or out of line, it
+// cost the teams up to 8 % at 5 digits.
 template <int S>
 struct ChunkShared {
   double X[32][33];                              // the solved block: [row][live column]
@@ -607,7 +607,7 @@ struct ChunkShared {
 };
 
 template <int S>
-__device__ __noinline__ void trsm_chunk(const PlanPtrs &P, int task, const double *__restrict__ Lv, const double *__restrict__ invd,
+__device__ __forceinline__ void trsm_chunk(const PlanPtrs &P, int task, const double *__restrict__ Lv, const double *__restrict__ invd,
                            const TrsmSplit &sp, double *__restrict__ Y, ChunkShared<S> &sm, bool unscaled) {
   const TrsmTask t = P.trsm_tasks[task];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -792,14 +792,10 @@ __device__ __noinline__ void trsm_chunk(const PlanPtrs &P, int task, const doubl
 template <int C, int S>
 __global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(const PlanPtrs P, const double *__restrict__ Lv,
                                                               const double *__restrict__ invd, const TrsmSplit sp,
-                                                              double *__restrict__ Y, int n_team) {
+                                                              double *__restrict__ Y) {
   extern __shared__ __align__(16) unsigned char team_smem[];
   constexpr int kParts = kChunk / (4 * C);
-  if ((int)blockIdx.x >= n_team) {                                 // a CTA per task behind them
-    if (*sp.unscaled) trsm_chunk<S>(P, (int)blockIdx.x - n_team, Lv, invd, sp, Y, *reinterpret_cast<ChunkShared<S> *>(team_smem), true);
-    return;
-  }
-  if (*sp.unscaled) return;
+  if (*sp.unscaled) return;                                        // trsm_chunk_kernel takes the launch over
   trsm_team<C, S>(P, P.trsm_tasks[blockIdx.x / kParts], blockIdx.x % kParts, Lv, invd, sp, Y,
                   *reinterpret_cast<TeamShared<C, S> *>(team_smem), threadIdx.x >> 5, threadIdx.x & 31);
 }
@@ -807,9 +803,10 @@ __global__ void __launch_bounds__(kThreads, C >= 4 ? 4 : 3) trsm_split_kernel(co
 template <int S>
 __global__ void __launch_bounds__(kThreads, S <= 4 ? 6 : S == 5 ? 5 : 4) trsm_chunk_kernel(const PlanPtrs P, const double *__restrict__ Lv,
                                                                  const double *__restrict__ invd, const TrsmSplit sp,
-                                                                 double *__restrict__ Y) {
+                                                                 double *__restrict__ Y, bool always) {
   __shared__ ChunkShared<S> sm;
-  trsm_chunk<S>(P, blockIdx.x, Lv, invd, sp, Y, sm, *sp.unscaled != 0);
+  const bool unscaled = *sp.unscaled != 0;
+  if (always || unscaled) trsm_chunk<S>(P, blockIdx.x, Lv, invd, sp, Y, sm, unscaled);
 }
 
 }  // namespace
@@ -841,9 +838,9 @@ int launch_lpack_split(const sc_ctx &c, int S_, int64_t base, int64_t count, con
 template <int C, int S>
 static void launch_team(const PlanPtrs &p, int n, const double *Lv, const double *invd, const TrsmSplit &sp, double *Y,
                         cudaStream_t st) {
-  const int smem = (int)std::max(sizeof(TeamShared<C, S>), sizeof(ChunkShared<S>)), n_team = n * (kChunk / (4 * C));
+  const int smem = (int)sizeof(TeamShared<C, S>);
   cudaFuncSetAttribute(trsm_split_kernel<C, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  trsm_split_kernel<C, S><<<(unsigned)(n_team + n), kThreads, smem, st>>>(p, Lv, invd, sp, Y, n_team);
+  trsm_split_kernel<C, S><<<(unsigned)(n * (kChunk / (4 * C))), kThreads, smem, st>>>(p, Lv, invd, sp, Y);
 }
 
 int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t count, const double *Lv,
@@ -860,7 +857,7 @@ int launch_trsm_split(const sc_ctx &c, int S_, int cols, int64_t base, int64_t c
 #define TS(S)                                                                                                   \
   if (cols == 2) launch_team<2, S>(p, (int)count, Lv, invd, sp, Y, st);                                         \
   else if (cols == 4) launch_team<4, S>(p, (int)count, Lv, invd, sp, Y, st);                                    \
-  else trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y)
+  trsm_chunk_kernel<S><<<(unsigned)count, kThreads, 0, st>>>(p, Lv, invd, sp, Y, cols >= 8)
   SC_SPLIT_SWITCH(S_, TS)
 #undef TS
   return (int)cudaGetLastError();

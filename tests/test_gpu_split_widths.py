@@ -34,8 +34,8 @@ def _width(plan):
 @pytest.mark.parametrize("digits,bound", [(7, 1e-12), (6, 5e-10), (5, 1.8e-9), (4, 4.7e-7), (3, 1.2e-4)])   # 2^(-8 S) times 2e3, or 1e-12
 def test_widths_agree(digits, bound):
     torch = pytest.importorskip("torch")
-    # separators of 147 columns, blocks of one to 32 columns, chunks of 32 and of 25 columns
-    subs = synth.elasticity_cubes((2, 2, 2), 6, 6, 1).subdomains[:2]
+    # 3000 dofs: separators of up to 300 columns, blocks of one to 32 columns, chunks of 32 and of 24 columns
+    subs = synth.elasticity_cubes((2, 2, 1), 9, 9, 1).subdomains[:1]
     fs = host.factorize_problem(subs)
     n_dual = 1 + max(int(f.lambda_map.max()) for f in fs)
 
@@ -50,16 +50,14 @@ def test_widths_agree(digits, bound):
     one, F1 = assemble(fs[:1])
     r, b = _width(one)
     assert r > 4                                              # two columns to a warp
-    some, Fs = assemble(fs * 12)
+    some, Fs = assemble(fs * 20)
     r, b = _width(some)
     assert r <= 4 and 300 * r > b                             # four
-    many, Fm = assemble(fs * 200)
+    many, Fm = assemble(fs * 100)
     r, b = _width(many)
-    assert 300 * r <= b and r <= 1                            # the whole chunk
+    assert max(300 * r, 180) <= b and r <= 1                  # the whole chunk
     n = int(one.F_offsets[1])
-    assert torch.equal(F1[:n], Fs[:n]) and torch.equal(F1[:n], Fm[:n])
-    a = int(many.F_offsets[2])
-    assert torch.equal(Fs[:a], Fm[:a])
-    Fo = oracle.dual_operators(subs)
-    for i in range(len(fs)):
-        assert oracle.relative_frobenius(many.export(Fm, i).cpu().numpy(), Fo[i]) <= bound
+    for i in (0, 7, 19):
+        assert torch.equal(F1, Fs[i * n:(i + 1) * n]) and torch.equal(F1, Fm[i * n:(i + 1) * n])
+    Fo = oracle.dual_operators(subs, refine=1)
+    assert oracle.relative_frobenius(many.export(Fm, 99).cpu().numpy(), Fo[0]) <= bound
